@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "dslash.cuh"
+#include "quad.cuh"
 
 namespace swc {
 
@@ -126,12 +127,21 @@ struct SWOp {
   using Vec = VA<3>;
   G U;
   Wt W;
-  __device__ __forceinline__ CV<T, 3> apply(const Geom& g, int n, const Vec& in, T m, T r, bool dag) const {
-    const V3<T> o = sw_site<T>(g, n, U, W, in, m, r, dag);
-    CV<T, 3> v;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) v.c[i] = o.c[i];
-    return v;
+  // four-lane form (FP64) at every volume: 14 against 40 us (8^4 and below), 218
+  // against 245 (16^3x32), 1067 against 1178 (24^3x48) for an application
+  static constexpr int kQuadVolume = 1 << 28;
+  static constexpr int kOwn = 2;  // the real numbers lane q of a site owns
+  __device__ static __forceinline__ bool owns(int q, int k) { return k == 0 || !(q & 1); }
+  __device__ static __forceinline__ size_t own(int n, int q, int k) {
+    return ((size_t)n * 3 + ((q & 1) ? 1 : 2 * k)) * 2 + (q >> 1);
+  }
+  __device__ __forceinline__ void quad(const Geom& g, int n, int q, const Vec& in, double m, double r, bool dag,
+                                       double o[kOwn]) const {
+    double h[3];
+    sw_quad(g, n, q, U, W, in, r, dag, h);
+    const double* self = reinterpret_cast<const double*>(in.p);
+    o[0] = fma(r + m, __ldg(self + own(n, q, 0)), (q & 1) ? h[1] : h[0]);
+    o[1] = (q & 1) ? 0.0 : fma(r + m, __ldg(self + own(n, q, 1)), h[2]);
   }
   template <int NS, typename GG>
   __device__ __forceinline__ void apply_multi(const GG& g, int n, const Vec& in, size_t stride, unsigned act,
@@ -169,6 +179,26 @@ struct WOp {
   using Vec = VA<12>;
 
   G U;
+  // four-lane form (FP64): the full 4-spinor hops at every volume (1765 against
+  // 1964 us at 24^3x48); the spin-projected ones up to 7 2^14 sites (176 against
+  // 187 us at 16^3x24; one thread a site: 220 against 225 us at 16^3x32, 1064
+  // against 1111 at 24^3x48)
+  static constexpr int kQuadVolume = R1 ? 7 << 14 : 1 << 28;
+  static constexpr int kOwn = 6;
+  __device__ static __forceinline__ bool owns(int, int) { return true; }
+  __device__ static __forceinline__ size_t own(int n, int q, int k) { return ((size_t)n * 12 + 3 * q) * 2 + k; }
+  __device__ __forceinline__ void quad(const Geom& g, int n, int q, const Vec& in, double m, double r, bool dag,
+                                       double o[kOwn]) const {
+    cx<double> h[3];
+    wilson_quad<R1>(g, n, q, U, in, r, dag, h);
+    const double diag = 4.0 * r + m;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const cx<double> self = in.ld(n, 3 * q + i);
+      o[2 * i] = fma(diag, self.re, -0.5 * h[i].re);
+      o[2 * i + 1] = fma(diag, self.im, -0.5 * h[i].im);
+    }
+  }
   __device__ __forceinline__ CV<T, 12> apply(const Geom& g, int n, const Vec& in, T m, T r, bool dag) const {
     const Sp<T> o = wilson_site<T, R1>(g, n, U, in, m, r, dag);
     CV<T, 12> v;
@@ -368,6 +398,50 @@ __device__ __forceinline__ unsigned running_mask(const SysState* S, int sys0, in
   return act;
 }
 
+// ---------------------------------------------------------------- state updates
+// k1's: |t|^2 = <p, A p> -> alpha
+__device__ __forceinline__ void finish_k1(SysState& st, const RedBuf& rb, int sys, double pAp) {
+  st.pAp = pAp;
+  if (!(pAp > 0.0) || !isfinite(pAp)) {
+    st.status = ST_FAILED;
+  } else {
+    st.alpha = st.rr / pAp;
+    record(rb, sys, st.iter, 0, st.alpha);
+  }
+}
+// k2's: |r|^2 -> beta, and whether the system goes on
+__device__ __forceinline__ void finish_k2(SysState& st, const RedBuf& rb, int sys, double rr) {
+  st.iter += 1;
+  if (!isfinite(rr)) {
+    st.status = ST_FAILED;
+  } else {
+    st.rr_old = st.rr;
+    st.rr = rr;
+    st.beta = rr / st.rr_old;
+    record(rb, sys, st.iter - 1, 1, st.beta);
+    if (rr > st.rmax2) st.rmax2 = rr;
+    if (rr <= st.trig2 || st.iter >= st.max_iter || rr < st.delta2 * st.rmax2) st.status = ST_NEED_RU;
+  }
+}
+// the FP64 residual's: converged, out of iterations, or on with the new residual
+__device__ __forceinline__ void finish_residual(SysState& s, const RedBuf& rb, int sys, double rr) {
+  s.rr_true = rr;
+  s.n_ru += 1;
+  if (!isfinite(rr)) {
+    s.status = ST_FAILED;
+  } else if (rr <= s.tol2) {
+    s.status = ST_CONVERGED;
+  } else if (s.iter >= s.max_iter) {
+    s.status = ST_MAXITER;
+  } else {
+    s.beta = (s.iter == 0) ? 0.0 : rr / s.rr_old;
+    record(rb, sys, s.iter - 1, 1, s.beta);
+    s.rr = rr;
+    s.rmax2 = rr;
+    s.status = ST_JUST_UPDATED;
+  }
+}
+
 // ---------------------------------------------------------------- k1: t = D p, |t|^2
 // blockIdx.y = group of NS consecutive systems; tickets are per group.
 // nact (instrumentation, may be null): the systems this launch computes are
@@ -436,16 +510,7 @@ __global__ void __launch_bounds__(kTile, stencil_min_blocks<T, Op>()) cg_k1(GG g
       if (!(act & (1u << s))) continue;
       const int sys = sys0 + s;
       const double pAp = finalize_sum(rb, sys, kWarps * ntiles, sm);
-      if (threadIdx.x == 0) {
-        SysState& st = S[sys];
-        st.pAp = pAp;
-        if (!(pAp > 0.0) || !isfinite(pAp)) {
-          st.status = ST_FAILED;
-        } else {
-          st.alpha = st.rr / pAp;
-          record(rb, sys, st.iter, 0, st.alpha);
-        }
-      }
+      if (threadIdx.x == 0) finish_k1(S[sys], rb, sys, pAp);
     }
   }
 }
@@ -499,20 +564,7 @@ __global__ void __launch_bounds__(kTile, stencil_min_blocks<T, Op>()) cg_k2(GG g
       if (!(act & (1u << s))) continue;
       const int sys = sys0 + s;
       const double rr = finalize_sum(rb, sys, kWarps * ntiles, sm);
-      if (threadIdx.x == 0) {
-        SysState& st = S[sys];
-        st.iter += 1;
-        if (!isfinite(rr)) {
-          st.status = ST_FAILED;
-        } else {
-          st.rr_old = st.rr;
-          st.rr = rr;
-          st.beta = rr / st.rr_old;
-          record(rb, sys, st.iter - 1, 1, st.beta);
-          if (rr > st.rmax2) st.rmax2 = rr;
-          if (rr <= st.trig2 || st.iter >= st.max_iter || rr < st.delta2 * st.rmax2) st.status = ST_NEED_RU;
-        }
-      }
+      if (threadIdx.x == 0) finish_k2(S[sys], rb, sys, rr);
     }
   }
 }
@@ -680,6 +732,80 @@ __global__ void __launch_bounds__(kTile) residual64(Geom g, Op op, typename Op::
         s.rmax2 = rr;
         s.status = ST_JUST_UPDATED;
       }
+    }
+  }
+}
+
+// ---------------------------------------------------------------- four lanes a site (FP64)
+// The FP64 kernels above with the four-lane site form (quad.cuh), for lattices
+// that one thread a site does not fill the chip with; the same arguments, with
+// tiles of 32 sites.
+constexpr int kQuadSites = kTile / 4;
+
+template <typename Op>
+__global__ void __launch_bounds__(kTile) apply_quad(Geom g, Op op, typename Op::Vec in, typename Op::Vec out,
+                                                  double mass0, size_t sstride, double r, int dagger,
+                                                  const SysState* S, int only_status, int* nact = nullptr,
+                                                  typename Op::Vec sub = {}, int has_sub = 0) {
+  const int sys = blockIdx.y, q = threadIdx.x & 3;
+  if (S && S[sys].status != only_status) return;
+  if (nact && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(nact, 1);
+  in = sys_view(in, sys, sstride);
+  out = sys_view(out, sys, sstride);
+  if (has_sub) sub = sys_view(sub, sys, sstride);
+  const double m = S ? S[sys].mass : mass0;
+  double* od = reinterpret_cast<double*>(out.p);
+  const double* sd = reinterpret_cast<const double*>(sub.p);
+  for (int n = blockIdx.x * kQuadSites + (threadIdx.x >> 2); n < g.V; n += gridDim.x * kQuadSites) {
+    double o[Op::kOwn];
+    op.quad(g, n, q, in, m, r, dagger != 0, o);
+#pragma unroll
+    for (int k = 0; k < Op::kOwn; ++k) {
+      const size_t j = Op::own(n, q, k);
+      if (Op::owns(q, k)) od[j] = has_sub ? __ldg(sd + j) - o[k] : o[k];
+    }
+  }
+}
+
+// KIND 1: k1 (out = (D+m) in, |out|^2); 2: k2 (r -= alpha (D+m)^+ in, |r|^2);
+// 3: residual64 (r = (D+m)^+ in, |r|^2, the convergence decision).
+template <int KIND, typename Op>
+__global__ void __launch_bounds__(kTile) iter_quad(Geom g, Op op, typename Op::Vec in, typename Op::Vec out,
+                                                 size_t in_stride, size_t out_stride, double r, SysState* S, RedBuf rb,
+                                                 int* nact) {
+  __shared__ double sm[32];
+  __shared__ int last;
+  const int sys = blockIdx.y, q = threadIdx.x & 3;
+  if (S[sys].status != (KIND == 3 ? ST_RU_PENDING : ST_RUNNING)) return;
+  if (nact && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(nact, 1);
+  in = sys_view(in, sys, in_stride);
+  out = sys_view(out, sys, out_stride);
+  const double m = S[sys].mass, alpha = KIND == 2 ? S[sys].alpha : 0.0;
+  double* od = reinterpret_cast<double*>(out.p);
+  const int ntiles = (g.V + kQuadSites - 1) / kQuadSites;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int n = tile * kQuadSites + (threadIdx.x >> 2);
+    double acc = 0.0;
+    if (n < g.V) {  // (8 sites a warp and V a multiple of 16: whole warps)
+      double o[Op::kOwn];
+      op.quad(g, n, q, in, m, r, KIND != 1, o);
+#pragma unroll
+      for (int k = 0; k < Op::kOwn; ++k) {
+        const size_t j = Op::own(n, q, k);
+        if (!Op::owns(q, k)) continue;
+        const double v = KIND == 2 ? fma(-alpha, o[k], od[j]) : o[k];
+        od[j] = v;
+        acc = fma(v, v, acc);
+      }
+    }
+    put_tile(rb, sys, tile, block_sum(acc, sm));
+  }
+  if (block_done(rb, sys, &last, gridDim.x)) {
+    const double v = finalize_sum(rb, sys, ntiles, sm);
+    if (threadIdx.x == 0) {
+      if constexpr (KIND == 1) finish_k1(S[sys], rb, sys, v);
+      else if constexpr (KIND == 2) finish_k2(S[sys], rb, sys, v);
+      else finish_residual(S[sys], rb, sys, v);
     }
   }
 }

@@ -50,7 +50,25 @@ template <class Op, class = void> struct two_pass : std::false_type {};
 template <class Op> struct two_pass<Op, std::void_t<decltype(Op::kTwoPass)>> : std::bool_constant<Op::kTwoPass> {};
 template <class Op> constexpr int f64_stride_factor() { return two_pass<Op>::value ? 2 : 1; }
 
-inline int grid_for(const void* kernel, int block, int V, int nsys, int cap) {
+// The FP64 kernels with four lanes a site (quad.cuh) for lattices up to the
+// operator's kQuadVolume sites (by the volume only, so that a system's
+// arithmetic does not depend on its batch); operators without that form never.
+template <class Op> constexpr bool has_quad() { return !two_pass<Op>::value; }
+template <class Op> constexpr bool quad_always() {  // every volume the library takes
+  if constexpr (has_quad<Op>()) return Op::kQuadVolume >= 1 << 28;
+  return false;
+}
+template <class Op> bool use_quad(int V) {
+  if constexpr (has_quad<Op>()) return V <= Op::kQuadVolume;
+  return false;
+}
+constexpr int kOver64 = 8;  // waves of blocks of the FP64 kernels
+
+// over: waves of blocks at most.  Kernels bound by the FP64 pipe take several:
+// blocks that share the pipe do not run in rounds, and a block that loops over
+// tiles would leave the last of them to a few SMs (8^3x16, 12 systems: 256
+// tiles a system on 63 blocks are 5 rounds for 4.06).
+inline int grid_for(const void* kernel, int block, long long V, int nsys, int cap, int over = 1) {
   static std::mutex mu;
   static std::unordered_map<const void*, int> cache;
   int nb;
@@ -65,11 +83,15 @@ inline int grid_for(const void* kernel, int block, int V, int nsys, int cap) {
       nb = it->second;
     }
   }
-  int gx = (sm_count() * nb) / (nsys > 0 ? nsys : 1);
+  int gx = (sm_count() * nb * over) / (nsys > 0 ? nsys : 1);
   if (gx < 1) gx = 1;
-  const int need = (V + block - 1) / block;
-  if (gx > need) gx = need;
+  const long long need = (V + block - 1) / block;
+  if (gx > need) gx = (int)need;
   if (gx > cap) gx = cap;
+  if (over > 1) {  // even rounds
+    const long long rounds = (need + gx - 1) / gx;
+    gx = (int)((need + rounds - 1) / rounds);
+  }
   return gx;
 }
 
@@ -487,7 +509,7 @@ class Engine {
         reliable_update(n_ru, side_);
         cudaEventRecord(ev_join_, side_);
       } else {
-        reliable_update(n_ru, st_);
+        reliable_update(n_ru, st_, kOver64);
       }
     }
     if (run) {
@@ -697,15 +719,45 @@ class Engine {
       FpSample* fs = fp_sample(1, st_);
       if (prof()) prof_count(cls_rhs(), 1);
       prepass(opd_, V64{chi_}, s64_, ST_ADMIT, true, st_);
-      apply_kernel<double, OpD><<<dim3(grid_of((const void*)apply_kernel<double, OpD>, kTile, na), cap_), kTile,
-                                  0, st_>>>(g_, opd_, V64{chi_}, V64{ws_.b64}, 0.0, s64_, r_, 1, S, ST_ADMIT,
-                                            fs ? fs->cnt : nullptr);
+      apply64(V64{chi_}, V64{ws_.b64}, 1, na, ST_ADMIT, st_, fs ? fs->cnt : nullptr, V64{}, 0, kOver64);
       if (fs) cudaEventRecord(fs->e1, st_);
       norm_b<NC><<<dim3(gn, cap_), kTile, 0, st_>>>(g_.V, ws_.b64, x_, s64_, S, rb_);
       admit_vectors<NC><<<dim3(gv, cap_), 256, 0, st_>>>(g_.V, x_, ws_.r64, ws_.b64, s64_, S);
     }
     admit_states<<<(cap_ + 127) / 128, 128, 0, st_>>>(cap_, S, MIXED ? 1 : 0);
     launches(5);
+  }
+
+  // (D+m) or its adjoint in FP64 on the systems in `status`; has_sub: sub - that.
+  void apply64(V64 in, V64 out, int dagger, int nsys, int status, cudaStream_t sx, int* cnt, V64 sub, int has_sub,
+               int over) {
+    if constexpr (has_quad<OpD>())
+      if (use_quad<OpD>(g_.V)) {
+        const int gx = grid_of((const void*)apply_quad<OpD>, kTile, nsys, 4, over);
+        apply_quad<OpD><<<dim3(gx, cap_), kTile, 0, sx>>>(g_, opd_, in, out, 0.0, s64_, r_, dagger, ws_.S, status,
+                                                          cnt, sub, has_sub);
+        return;
+      }
+    if constexpr (!quad_always<OpD>()) {
+      const int gx = grid_of((const void*)apply_kernel<double, OpD>, kTile, nsys, 1, over);
+      apply_kernel<double, OpD><<<dim3(gx, cap_), kTile, 0, sx>>>(g_, opd_, in, out, 0.0, s64_, r_, dagger, ws_.S,
+                                                                  status, cnt, sub, has_sub);
+    }
+  }
+
+  // r64 = (D+m)^+ t64 and the convergence decisions (systems in RU_PENDING).
+  void residual(int nsys, cudaStream_t sx, int over) {
+    if constexpr (has_quad<OpD>())
+      if (use_quad<OpD>(g_.V)) {
+        const int gx = grid_of((const void*)iter_quad<3, OpD>, kTile, nsys, 4, over);
+        iter_quad<3, OpD><<<dim3(gx, cap_), kTile, 0, sx>>>(g_, opd_, V64{ws_.t64}, V64{ws_.r64}, s64_, s64_, r_, ws_.S,
+                                                            rbu_, nullptr);
+        return;
+      }
+    if constexpr (!quad_always<OpD>()) {
+      const int gx = grid_of((const void*)residual64<OpD>, kTile, nsys, 1, over);
+      residual64<OpD><<<dim3(gx, cap_), kTile, 0, sx>>>(g_, opd_, V64{ws_.t64}, V64{ws_.r64}, bp_, ws_.S, rbu_);
+    }
   }
 
   // Device address of a host status buffer that is pinned and mapped, else
@@ -753,7 +805,10 @@ class Engine {
 
   // The reliable update of the systems in RU_PENDING, on stream `sx`.
   // nsys: the slots (at most) that take the update this round, for the grids.
-  void reliable_update(int nsys, cudaStream_t sx) {
+  // over: waves of blocks of the FP64 kernels; 1 where iterations run beside
+  // them (with 8 the queued FP64 blocks hold the SMs against them: 48 Wilson
+  // systems at 16^3x32 274 against 270 ms).
+  void reliable_update(int nsys, cudaStream_t sx, int over = 1) {
     SysState* S = ws_.S;
     const int gv = grid_of((const void*)cg_k3<TF, VR, VF, NC>, 256, nsys);
     const int g3 = grid_of(k3_ptr(), 256, k3_rows(nsys));
@@ -764,12 +819,9 @@ class Engine {
     if (prof()) prof_count(cls_ru(), 1);
     // r = (D+m)^+ (chi - (D+m) x) = b - A x, all in FP64
     prepass(opd_, V64{x_}, s64_, ST_RU_PENDING, false, sx);
-    apply_kernel<double, OpD><<<dim3(grid_of((const void*)apply_kernel<double, OpD>, kTile, nsys), cap_), kTile, 0,
-                                sx>>>(g_, opd_, V64{x_}, V64{ws_.t64}, 0.0, s64_, r_, 0, S, ST_RU_PENDING,
-                                      fs ? fs->cnt : nullptr, V64{chi_}, 1);
+    apply64(V64{x_}, V64{ws_.t64}, 0, nsys, ST_RU_PENDING, sx, fs ? fs->cnt : nullptr, V64{chi_}, 1, over);
     prepass(opd_, V64{ws_.t64}, s64_, ST_RU_PENDING, true, sx);
-    residual64<OpD><<<dim3(grid_of((const void*)residual64<OpD>, kTile, nsys), cap_), kTile, 0, sx>>>(
-        g_, opd_, V64{ws_.t64}, V64{ws_.r64}, bp_, S, rbu_);
+    residual(nsys, sx, over);
     if (fs) cudaEventRecord(fs->e1, sx);
     if constexpr (MIXED) demote_r<NC, VR><<<dim3(gv, cap_), 256, 0, sx>>>(gb_, ws_.r64, fr_, s64_, runits_, S);
     launch_k3(g3, ST_JUST_UPDATED, 2, sx, nullptr);
@@ -816,8 +868,15 @@ class Engine {
   // run (blocks of stopped slots return at once).
   void set_grids(int groups) {
     cls_ = groups;
-    g1_ = grid_for(k1_ptr(), kTile, g_.V, groups, ntiles_);
-    g2_ = grid_for(k2_ptr(), kTile, g_.V, groups, ntiles_);
+    if (MIXED || !use_quad<OpF>(g_.V)) {
+      if constexpr (MIXED || !quad_always<OpF>()) {
+        g1_ = grid_for(k1_ptr(), kTile, g_.V, groups, ntiles_, MIXED ? 1 : kOver64);
+        g2_ = grid_for(k2_ptr(), kTile, g_.V, groups, ntiles_, MIXED ? 1 : kOver64);
+      }
+    } else if constexpr (!MIXED && has_quad<OpF>()) {
+      g1_ = grid_for((const void*)iter_quad<1, OpF>, kTile, 4LL * g_.V, groups, ntiles_ * 4, kOver64);
+      g2_ = grid_for((const void*)iter_quad<2, OpF>, kTile, 4LL * g_.V, groups, ntiles_ * 4, kOver64);
+    }
     gV_ = grid_for(k3_ptr(), 256, g_.V, k3_rows(groups * ns_), ntiles_);
   }
 
@@ -906,7 +965,14 @@ class Engine {
       else if (ns_ == 4) launch_k12<4>(c);
       else launch_k12<1>(c);
     } else {
-      launch_k12<1>(c);
+      if (!use_quad<OpF>(g_.V)) {
+        if constexpr (!quad_always<OpF>()) launch_k12<1>(c);
+      } else if constexpr (has_quad<OpF>()) {
+        iter_quad<1, OpF><<<dim3(g1_, cap_), kTile, 0, ist_>>>(g_, opf_, fp_, ft_, vunits_, vunits_, r_, S, rb_, c);
+        if (c) cudaEventRecord(samples_.back().e1, ist_);
+        iter_quad<2, OpF><<<dim3(g2_, cap_), kTile, 0, ist_>>>(g_, opf_, ft_, fr_, vunits_, runits_, r_, S, rb_,
+                                                               c ? c + 1 : nullptr);
+      }
     }
     if (sample) cudaEventRecord(samples_.back().e2, ist_);
     launch_k3(gV_, ST_RUNNING, 3, ist_, c ? c + 2 : nullptr);
@@ -973,8 +1039,10 @@ class Engine {
       cg_k3<TF, VR, VF, NC><<<dim3(gx, cap_), 256, 0, s>>>(g_.V, fr_, fp_, fx_, runits_, vunits_, ws_.S, status,
                                                            mode, nact);
   }
-  int grid_of(const void* kernel, int block, int nsys) const {
-    return grid_for(kernel, block, g_.V, nsys < 1 ? 1 : (nsys > cap_ ? cap_ : nsys), ntiles_);
+  // (lanes: threads a site)
+  int grid_of(const void* kernel, int block, int nsys, int lanes = 1, int over = 1) const {
+    return grid_for(kernel, block, (long long)g_.V * lanes, nsys < 1 ? 1 : (nsys > cap_ ? cap_ : nsys), ntiles_ * lanes,
+                    over);
   }
   int nrun_ = 0, ns_ = 1, gfast_ = 0;
   std::vector<Sample> samples_;

@@ -64,57 +64,6 @@ __device__ __forceinline__ void mdv_acc(V3<T>& acc, const M3<T>& M, const V3<T>&
     }
 }
 
-template <typename T, typename G, typename Wt, typename In>
-__device__ __forceinline__ V3<T> sw_site(const Geom& g, int n, const G& U, const Wt& W, const In& in,
-                                         T mass, T r, bool dagger) {
-  int x[4], df[4], db[4];
-  coords(g, n, x);
-  hop_deltas(g, n, x, df, db);
-  // st = sum_mu eta_mu [U_mu(x) psi(x+mu) - U_mu(x-mu)^+ psi(x-mu)]
-  V3<T> st = zero3<T>();
-  int par = 0;
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    V3<T> pf = ld3<In, T>(in, n + df[mu]), pb = ld3<In, T>(in, n + db[mu]);
-    if (mu == 3) {
-      if (bc_flip(g, x, +1)) neg3(pf);
-      if (bc_flip(g, x, -1)) neg3(pb);
-    }
-    if (mu == 0) {  // eta_0 = +1
-      mv_acc(st, U.link(n, mu), pf);
-      mdv_acc(st, U.link(n + db[mu], mu), pb, T(-1));
-    } else {
-      V3<T> d = zero3<T>();
-      mv_acc(d, U.link(n, mu), pf);
-      mdv_acc(d, U.link(n + db[mu], mu), pb, T(-1));
-      const T eta = (par & 1) ? T(-1) : T(1);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) st.c[i] = st.c[i] + eta * d.c[i];
-    }
-    par += x[mu];
-  }
-  // h = sum over the 16 corners of W(x,s) psi(x+s)
-  V3<T> h = zero3<T>();
-  const bool fflip = bc_flip(g, x, +1), bflip = bc_flip(g, x, -1);
-#pragma unroll 2
-  for (int k = 0; k < 8; ++k) {
-    int of, ob;
-    corner_offsets(k, df, db, of, ob);
-    V3<T> pf = ld3<In, T>(in, n + of), pb = ld3<In, T>(in, n + ob);
-    if (fflip) neg3(pf);
-    if (bflip) neg3(pb);
-    mv_acc(h, W.mat(n, k), pf);
-    mdv_acc(h, W.mat(n + ob, k), pb, T(1));
-  }
-  const T hs = (eps_eta5_neg(x) ? r : -r) * T(0.0625);
-  const T ss = dagger ? T(-0.5) : T(0.5);
-  const V3<T> self = ld3<In, T>(in, n);
-  V3<T> o;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) o.c[i] = ss * st.c[i] + (r + mass) * self.c[i] + hs * h.c[i];
-  return o;
-}
-
 template <typename T> struct Sp { V3<T> s[4]; };
 
 template <typename In, typename T> struct SpLoader {
@@ -194,6 +143,39 @@ __device__ __forceinline__ void wgeneral(int mu, T c, T r, const Sp<T>& f, Sp<T>
   }
 }
 
+// Both spin-projected hops of direction mu (r = 1): acc += (1 - c g_mu) Uf pf +
+// (1 + c g_mu) Ub^+ pb, boundary signs ff, fb.  With uf, ub the transported
+// rows, the upper spins take S = uf + ub and the lower ones the phase of
+// D = uf - ub = 2 uf - S: S continues uf's chain of FMAs, so a direction takes
+// 204 instructions of the FP64 pipe, which bounds the FP64 operators, where
+// two separate reconstructions take 216.
+template <typename T>
+__device__ __forceinline__ void wilson_mu(int mu, T c, const M3<T>& Uf, const M3<T>& Ub, const Sp<T>& pf,
+                                          const Sp<T>& pb, bool ff, bool fb, Sp<T>& acc) {
+  V3<T> h0, h1;
+  wproject(mu, c, pf, h0, h1);
+  V3<T> u0 = mv(Uf, h0), u1 = mv(Uf, h1);
+  if (ff) { neg3(u0); neg3(u1); }
+  V3<T> s0 = u0, s1 = u1;
+  wproject(mu, -c, pb, h0, h1);
+  if (fb) { neg3(h0); neg3(h1); }
+  mdv_acc(s0, Ub, h0, T(1));
+  mdv_acc(s1, Ub, h1, T(1));
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    acc.s[0].c[i] = acc.s[0].c[i] + s0.c[i];
+    acc.s[1].c[i] = acc.s[1].c[i] + s1.c[i];
+    const cx<T> d0 = {fma(T(2), u0.c[i].re, -s0.c[i].re), fma(T(2), u0.c[i].im, -s0.c[i].im)};
+    const cx<T> d1 = {fma(T(2), u1.c[i].re, -s1.c[i].re), fma(T(2), u1.c[i].im, -s1.c[i].im)};
+    switch (mu) {
+      case 0: acc.s[2].c[i] = acc.s[2].c[i] + c * times_i(d1); acc.s[3].c[i] = acc.s[3].c[i] + c * times_i(d0); break;
+      case 1: acc.s[2].c[i] = acc.s[2].c[i] - c * d1;          acc.s[3].c[i] = acc.s[3].c[i] + c * d0;          break;
+      case 2: acc.s[2].c[i] = acc.s[2].c[i] + c * times_i(d0); acc.s[3].c[i] = acc.s[3].c[i] - c * times_i(d1); break;
+      default: acc.s[2].c[i] = acc.s[2].c[i] - c * d0;         acc.s[3].c[i] = acc.s[3].c[i] - c * d1;          break;
+    }
+  }
+}
+
 template <typename T, bool R1, typename G, typename In>
 __device__ __forceinline__ Sp<T> wilson_site(const Geom& g, int n, const G& U, const In& in,
                                              T mass, T r, bool dagger) {
@@ -207,26 +189,11 @@ __device__ __forceinline__ Sp<T> wilson_site(const Geom& g, int n, const G& U, c
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     const int nf = n + df[mu], nb = n + db[mu];
-    T bf = T(1), bb = T(1);
-    if (mu == 3) {
-      if (bc_flip(g, x, +1)) bf = T(-1);
-      if (bc_flip(g, x, -1)) bb = T(-1);
-    }
+    const bool ff = mu == 3 && bc_flip(g, x, +1), fb = mu == 3 && bc_flip(g, x, -1);
     const M3<T> Uf = U.link(n, mu);
     const M3<T> Ub = U.link(nb, mu);
     if (R1) {
-      V3<T> h0, h1;
-      const Sp<T> pf = ld_sp<In, T>(in, nf);
-      wproject(mu, sg, pf, h0, h1);
-      V3<T> u0 = mv(Uf, h0), u1 = mv(Uf, h1);
-      if (bf < T(0)) { neg3(u0); neg3(u1); }
-      wreconstruct(mu, sg, u0, u1, acc);
-      const Sp<T> pb = ld_sp<In, T>(in, nb);
-      wproject(mu, -sg, pb, h0, h1);
-      u0 = mdv(Ub, h0);
-      u1 = mdv(Ub, h1);
-      if (bb < T(0)) { neg3(u0); neg3(u1); }
-      wreconstruct(mu, -sg, u0, u1, acc);
+      wilson_mu(mu, sg, Uf, Ub, ld_sp<In, T>(in, nf), ld_sp<In, T>(in, nb), ff, fb, acc);
     } else {
       const Sp<T> pf = ld_sp<In, T>(in, nf), pb = ld_sp<In, T>(in, nb);
       Sp<T> f, b;
@@ -234,8 +201,8 @@ __device__ __forceinline__ Sp<T> wilson_site(const Geom& g, int n, const G& U, c
       for (int s = 0; s < 4; ++s) {
         f.s[s] = mv(Uf, pf.s[s]);
         b.s[s] = mdv(Ub, pb.s[s]);
-        if (bf < T(0)) neg3(f.s[s]);
-        if (bb < T(0)) neg3(b.s[s]);
+        if (ff) neg3(f.s[s]);
+        if (fb) neg3(b.s[s]);
       }
       wgeneral(mu, sg, r, f, acc);
       wgeneral(mu, -sg, r, b, acc);

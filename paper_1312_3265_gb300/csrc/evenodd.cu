@@ -67,6 +67,11 @@ __device__ __forceinline__ Sp<T> wilson_hops(const Geom& g, int n, const int x[4
   for (int mu = 0; mu < 4; ++mu) {
     const int nf = hop(g, n, x, mu, +1), nb = hop(g, n, x, mu, -1);
     const bool ff = (mu == 3) && bc_flip(g, x, +1), fb = (mu == 3) && bc_flip(g, x, -1);
+    if constexpr (R1 && sizeof(T) == 8) {
+      wilson_mu(mu, sg, U.link(n, mu), U.link(nb, mu), ld_sp<In, T>(in, HALF ? (nf >> 1) : nf),
+                ld_sp<In, T>(in, HALF ? (nb >> 1) : nb), ff, fb, acc);
+      continue;
+    }
     {
       const M3<T> Uf = U.link(n, mu);
       const Sp<T> p = ld_sp<In, T>(in, HALF ? (nf >> 1) : nf);

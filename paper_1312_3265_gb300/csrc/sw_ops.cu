@@ -10,10 +10,8 @@ using SW16 = SWOp<float, GaugeP16, TransP16, VecP16>;
 int sw_apply_f64(const Geom& g, const double2* U, const double2* W, const double2* in, double2* out,
                  double mass, double r, int dagger, cudaStream_t st) {
   const SW64 op{GaugeC64{U}, TransC64{W}};
-  const int gx = (g.V + 127) / 128;
-  apply_kernel<double, SW64><<<dim3(gx, 1), 128, 0, st>>>(g, op, VecC64<3>{const_cast<double2*>(in)},
-                                                          VecC64<3>{out}, mass, 0, r, dagger,
-                                                          nullptr, 0);
+  const VecC64<3> vi{const_cast<double2*>(in)}, vo{out};
+  apply_quad<SW64><<<(g.V + kQuadSites - 1) / kQuadSites, kTile, 0, st>>>(g, op, vi, vo, mass, 0, r, dagger, nullptr, 0);
   note_launches(1);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SW_OK : cuda_fail(e);

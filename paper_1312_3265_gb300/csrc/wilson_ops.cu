@@ -13,10 +13,14 @@ template <bool R1>
 static int apply_impl(const Geom& g, const double2* U, const double2* in, double2* out, double mass, double r,
                       int dagger, cudaStream_t st) {
   const W64<R1> op{GaugeC64{U}};
-  const int gx = (g.V + 127) / 128;
-  apply_kernel<double, W64<R1>><<<dim3(gx, 1), 128, 0, st>>>(g, op, VecC64<12>{const_cast<double2*>(in)},
-                                                             VecC64<12>{out}, mass, 0, r, dagger,
-                                                             nullptr, 0);
+  const VecC64<12> vi{const_cast<double2*>(in)}, vo{out};
+  if (use_quad<W64<R1>>(g.V)) {
+    apply_quad<W64<R1>><<<(g.V + kQuadSites - 1) / kQuadSites, kTile, 0, st>>>(g, op, vi, vo, mass, 0, r, dagger,
+                                                                             nullptr, 0);
+  } else if constexpr (!quad_always<W64<R1>>()) {
+    apply_kernel<double, W64<R1>><<<(g.V + kTile - 1) / kTile, kTile, 0, st>>>(g, op, vi, vo, mass, 0, r, dagger,
+                                                                             nullptr, 0);
+  }
   note_launches(1);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SW_OK : cuda_fail(e);
