@@ -234,16 +234,24 @@ __device__ __forceinline__ void st_site(const Vec& v, int n, const CV<T, NC>& a)
 }
 template <int NC>
 __device__ __forceinline__ void st_site(const VecP16<NC>& v, int n, const CV<float, NC>& a) {
-  float m = 0.f;
+  float m = 0.f, inv;
 #pragma unroll
   for (int c = 0; c < NC; ++c) m = fmaxf(m, fmaxf(fabsf(a.c[c].re), fabsf(a.c[c].im)));
-  // Sites below 1e-30 (far tails of point-source solutions reach FP32
-  // denormals, whose reciprocal overflows) are stored as exact zeros.
-  if (!(m > 1e-30f)) m = (m == m) ? 0.f : m;
-  const float inv = m > 0.f ? 1.f / m : 0.f;
+  half_scale(m, inv);
+  unsigned u[NC];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) v.p[pk(n, NC, c)] = __floats2half2_rn(a.c[c].re * inv, a.c[c].im * inv);
-  reinterpret_cast<float*>(v.p + (size_t)NC * v.V)[n] = m;
+  for (int c = 0; c < NC; ++c) {
+    const __half2 h = __floats2half2_rn(a.c[c].re * inv, a.c[c].im * inv);
+    memcpy(&u[c], &h, 4);
+  }
+  uint4* b = reinterpret_cast<uint4*>(v.p);
+  if constexpr (NC == 3) {
+    b[n] = make_uint4(u[0], u[1], u[2], __float_as_uint(m));
+  } else {
+#pragma unroll
+    for (int q = 0; q < NC / 4; ++q) b[pk(n, NC / 4, q)] = make_uint4(u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+    v.scale(n) = m;
+  }
 }
 
 template <int NC>
@@ -276,17 +284,33 @@ template <int NC> struct SiteLoad<VecP32q<NC>> {
     return a;
   }
 };
+template <> struct SiteLoad<VecP16<12>> {
+  template <typename T, int N> static __device__ __forceinline__ CV<float, 12> ld(const VecP16<12>& v, int n) {
+    const Sp<float> p = ld_sp<VecP16<12>, float>(v, n);
+    CV<float, 12> a;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) a.c[c] = p.s[c / 3].c[c % 3];
+    return a;
+  }
+};
+template <> struct SiteLoad<VecP16<3>> {
+  template <typename T, int N> static __device__ __forceinline__ CV<float, 3> ld(const VecP16<3>& v, int n) {
+    const V3<float> p = ld3<VecP16<3>, float>(v, n);
+    return {{p.c[0], p.c[1], p.c[2]}};
+  }
+};
 template <typename T, int NC, typename Vec> __device__ __forceinline__ CV<T, NC> ld_site(const Vec& v, int n) {
   return SiteLoad<Vec>::template ld<T, NC>(v, n);
 }
 
 // FP32 residual / solution storage that goes with a stencil storage: the
-// Wilson float4 planes keep r and x in float4 planes too (the r update of k2
+// Wilson storages keep r and x in float4 planes (the r update of k2
 // and the streaming k3 then move whole sites in 16-byte units, half the
 // memory instructions of float2 planes); every other storage pairs with plain
 // float2 planes.
 template <typename VF, int NC> struct RVecOf { using type = VecP32<NC>; };
 template <> struct RVecOf<VecP32q<12>, 12> { using type = VecP32q<12>; };
+template <> struct RVecOf<VecP16<12>, 12> { using type = VecP32q<12>; };
 
 // Per-system view of a batched vector: system `sys` starts `sys * sstride`
 // complex numbers after the base pointer (layout inside a system unchanged).

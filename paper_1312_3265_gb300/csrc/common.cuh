@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -350,6 +351,10 @@ struct TransP32 {
   }
 };
 
+// Sites a packed field has room for: whole groups (half-lattice fields may end
+// in a partial one).
+__host__ __device__ __forceinline__ size_t padded(int V) { return ((size_t)V + 15) & ~(size_t)15; }
+
 // Vector fields: NC complex components per site.
 template <int NC> struct VecC64 {  // canonical [V][NC] complex128
   using unit = double2;
@@ -360,7 +365,7 @@ template <int NC> struct VecC64 {  // canonical [V][NC] complex128
 };
 template <int NC> struct VecP32 {  // packed, NC float2 planes
   using unit = float2;
-  static size_t sys_units(int V) { return (size_t)V * NC; }
+  static size_t sys_units(int V) { return padded(V) * NC; }
   float2* p;
   int V;  // volume (the packed addressing itself needs only n)
   __device__ __forceinline__ cx<float> ld(int n, int c) const { float2 v = __ldg(p + pk(n, NC, c)); return {v.x, v.y}; }
@@ -373,7 +378,7 @@ template <int NC> struct VecP32 {  // packed, NC float2 planes
 template <int NC> struct VecP32q {
   static_assert(NC % 2 == 0, "pairs of components");
   using unit = float4;
-  static size_t sys_units(int V) { return (size_t)V * NC / 2; }
+  static size_t sys_units(int V) { return padded(V) * NC / 2; }
   float4* p;
   int V;  // volume (the packed addressing itself needs only n)
   __device__ __forceinline__ cx<float> ld(int n, int c) const {
@@ -395,7 +400,7 @@ template <int NC> struct VecP32q {
 template <int NC> struct VecP32x2 {
   using unit = float4;
   static constexpr bool kPaired = true;
-  static size_t sys_units(int V) { return (size_t)V * NC / 2; }
+  static size_t sys_units(int V) { return padded(V) * NC / 2; }
   float4* p;
   int V;  // volume (the packed addressing itself needs only n)
   int lane = 0;
@@ -434,12 +439,18 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return make_float2
 //          (24 planes); the third row is rebuilt as conj(row0 x row1), exact
 //          for SU(3) links
 //   transports: all 9 entries, 72 half2 planes (not unitary: no compression)
-//   vectors: NC half2 planes holding psi/scale, then one float scale per site
-//          (the largest |re|, |im| of the site, site-major), so every site
-//          keeps FP16's relative precision whatever its magnitude
+//   vectors: half2 components holding psi/scale and one float scale per site
+//          (the largest |re|, |im| of the site), so every site keeps FP16's
+//          relative precision whatever its magnitude
 __device__ __forceinline__ cx<float> h2c(__half2 h) {
   const float2 f = __half22float2(h);
   return {f.x, f.y};
+}
+
+__device__ __forceinline__ cx<float> half2_of(unsigned u) {  // a half2 by its bits
+  __half2 h;
+  memcpy(&h, &u, 4);
+  return h2c(h);
 }
 
 // row 2 of an SU(3) matrix from rows 0 and 1: conj(row0 x row1)
@@ -487,23 +498,56 @@ struct TransP16 {
     return M;
   }
 };
-template <int NC> struct VecP16 {  // per system: NC packed half2 planes, then [V] float scales
+// scale and reciprocal of an FP16 site from its largest |re|, |im| (sites
+// below 1e-30 -- far tails of point-source solutions reach FP32 denormals,
+// whose reciprocal overflows -- are stored as exact zeros)
+__device__ __forceinline__ void half_scale(float& m, float& inv) {
+  if (!(m > 1e-30f)) m = (m == m) ? 0.f : m;
+  inv = m > 0.f ? 1.f / m : 0.f;
+}
+template <int NC> struct VecP16;
+// spinors: 3 planes of 16-byte units, plane k holding components 4k .. 4k + 3
+// (a whole site moves in three 16-byte loads), then one float scale per site
+template <> struct VecP16<12> {
   using unit = __half2;
-  static size_t sys_units(int V) { return (size_t)V * (NC + 1); }
+  static size_t sys_units(int V) { return padded(V) * 13; }
   __half2* p;
   int V;
-  __device__ __forceinline__ const float* sc() const { return reinterpret_cast<const float*>(p + (size_t)NC * V); }
+  __device__ __forceinline__ const float* sc() const { return reinterpret_cast<const float*>(p + 12 * padded(V)); }
+  __device__ __forceinline__ float& scale(int n) const { return reinterpret_cast<float*>(p + 12 * padded(V))[n]; }
+  __device__ __forceinline__ __half2* at(int n, int c) const { return p + pk(n, 3, c >> 2) * 4 + (c & 3); }
   __device__ __forceinline__ cx<float> ld(int n, int c) const {
-    const cx<float> v = h2c(__ldg(p + pk(n, NC, c)));
+    const cx<float> v = h2c(__ldg(at(n, c)));
     const float s = __ldg(sc() + n);
+    return {v.re * s, v.im * s};
+  }
+};
+// colour vectors: one 16-byte unit per site, three half2 and the float scale
+template <> struct VecP16<3> {
+  using unit = __half2;
+  static size_t sys_units(int V) { return padded(V) * 4; }
+  __half2* p;
+  int V;
+  __device__ __forceinline__ float& scale(int n) const { return reinterpret_cast<float*>(p)[(size_t)n * 4 + 3]; }
+  __device__ __forceinline__ __half2* at(int n, int c) const { return p + (size_t)n * 4 + c; }
+  __device__ __forceinline__ cx<float> ld(int n, int c) const {
+    const cx<float> v = h2c(__ldg(at(n, c)));
+    const float s = __ldg(reinterpret_cast<const float*>(p) + (size_t)n * 4 + 3);
     return {v.re * s, v.im * s};
   }
 };
 
 template <typename Acc, typename T> __device__ __forceinline__ V3<T> ld3(const Acc& a, int n, int off = 0) {
   V3<T> v;
+  if constexpr (std::is_same<Acc, VecP16<3>>::value) {  // one 16-byte load
+    const uint4 w = __ldg(reinterpret_cast<const uint4*>(a.p) + n);
+    const unsigned u[3] = {w.x, w.y, w.z};
 #pragma unroll
-  for (int i = 0; i < 3; ++i) v.c[i] = a.ld(n, off + i);
+    for (int i = 0; i < 3; ++i) v.c[i] = __uint_as_float(w.w) * half2_of(u[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v.c[i] = a.ld(n, off + i);
+  }
   return v;
 }
 

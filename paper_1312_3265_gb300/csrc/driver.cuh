@@ -28,6 +28,7 @@
 #include "internal.h"
 #include "misc_kernels.cuh"
 #include "ritz.h"
+#include "small.cuh"
 
 namespace swc {
 
@@ -192,6 +193,8 @@ struct Workspace {
   unsigned* tickets;  // [2 nsys]: iteration kernels, then reliable-update kernels
   double* mass;
   double* hist;  // CG coefficients, [nsys][kHist][2]
+  unsigned long long* slots;  // small lattices (small.cuh): tagged tile sums
+  int* list;     // the same: list of the running systems [cap + 1], "gave up" words [cap], barrier epochs
   int* pcount;   // systems computed per sampled launch: [kProfSlots/2][3] (k1, k2, k3), then the FP64 samples
   int* ctl;      // device-driven solve: [0] rounds run, [1] round cap reached
 };
@@ -211,17 +214,18 @@ inline size_t workspace_bytes_pt(int V, int NC, int nsys, bool mixed, size_t pt,
   const size_t n = (size_t)V * NC * nsys * f64_factor;
   const size_t ntiles = (size_t)(V + kTile - 1) / kTile;
   size_t b = (mixed ? 2 : 3) * align_up(sizeof(double2) * n);  // b64 only in FP64 mode
-  const size_t n32 = (size_t)V * NC * nsys;  // FP32 r and x carry no scratch
+  const size_t n32 = padded(V) * NC * nsys;  // FP32 r and x carry no scratch
   b += mixed ? 2 * align_up(pt * nsys_pt) + 2 * align_up(sizeof(float2) * n32) : align_up(pt * nsys_pt);
   b += align_up(sizeof(SysState) * nsys) + align_up(sizeof(double) * 2 * kWarps * ntiles * nsys) +
        align_up(sizeof(unsigned) * 2 * nsys) + align_up(sizeof(double) * nsys) +
+       (mixed ? align_up(8 * small_slots(V, nsys)) + align_up(sizeof(int) * small_words(V, nsys)) : 0) +
        align_up(sizeof(double) * 2 * kHist * nsys) + align_up(sizeof(int) * 2 * kProfSlots) +
        align_up(sizeof(int) * 8);
   return b;
 }
 // FP64 or FP32 storage of p and t
 inline size_t workspace_bytes(int V, int NC, int nsys, bool mixed) {
-  return workspace_bytes_pt(V, NC, nsys, mixed, (size_t)V * NC * (mixed ? sizeof(float2) : sizeof(double2)));
+  return workspace_bytes_pt(V, NC, nsys, mixed, mixed ? padded(V) * NC * sizeof(float2) : (size_t)V * NC * sizeof(double2));
 }
 // f64_factor: 2 for two-pass operators, whose FP64 vectors and stencil
 // vectors p, t carry their scratch after each system's field
@@ -235,7 +239,7 @@ inline Workspace carve_workspace_pt(void* base, int V, int NC, int nsys, bool mi
                                     int nsys_pt = -1) {
   if (nsys_pt < 0) nsys_pt = nsys;
   const size_t n = (size_t)V * NC * nsys * f64_factor;
-  const size_t n32 = (size_t)V * NC * nsys;
+  const size_t n32 = padded(V) * NC * nsys;
   const size_t ntiles = (size_t)(V + kTile - 1) / kTile;
   char* c = static_cast<char*>(base);
   auto take = [&](size_t bytes) {
@@ -260,6 +264,10 @@ inline Workspace carve_workspace_pt(void* base, int V, int NC, int nsys, bool mi
   w.partials = (double*)take(sizeof(double) * 2 * kWarps * ntiles * nsys);  // 2nd half: norm_b's |x0|^2
   w.tickets = (unsigned*)take(sizeof(unsigned) * 2 * nsys);  // 2nd half: the reliable-update kernels
   w.mass = (double*)take(sizeof(double) * nsys);
+  if (mixed) {
+    w.slots = (unsigned long long*)take(8 * small_slots(V, nsys));
+    w.list = (int*)take(sizeof(int) * small_words(V, nsys));
+  }
   w.hist = (double*)take(sizeof(double) * 2 * kHist * nsys);
   w.pcount = (int*)take(sizeof(int) * 2 * kProfSlots);
   w.ctl = (int*)take(sizeof(int) * 8);
@@ -267,7 +275,7 @@ inline Workspace carve_workspace_pt(void* base, int V, int NC, int nsys, bool mi
 }
 inline Workspace carve_workspace(void* base, int V, int NC, int nsys, bool mixed) {
   return carve_workspace_pt(base, V, NC, nsys, mixed,
-                            (size_t)V * NC * (mixed ? sizeof(float2) : sizeof(double2)));
+                            mixed ? padded(V) * NC * sizeof(float2) : (size_t)V * NC * sizeof(double2));
 }
 template <class PVec>
 inline Workspace carve_workspace_for(void* base, int V, int NC, int nsys, bool mixed, int f64_factor = 1) {
@@ -337,6 +345,25 @@ class Engine {
     ns_ = MIXED ? param_ns(NC) : 1;
     ngrp_ = (cap + ns_ - 1) / ns_;
     set_grids(ngrp_);
+    if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
+      small_ = small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
+      if (small_) {
+        for (int wide = 0; wide < (splan_.nt <= kSmallWide ? 2 : 1); ++wide) {
+          int nb = 0;
+          if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, small_kernel(opf_, wide != 0), splan_.nt, 0) !=
+              cudaSuccess)
+            nb = 0;
+          small_blocks_[wide] = nb * sm_count();
+        }
+        if (small_blocks_[0] < splan_.tiles) {
+          cudaGetLastError();
+          small_ = false;
+        } else {
+          cudaMemsetAsync(ws.slots, 0, 8 * small_slots(g.V, cap), st);
+          cudaMemsetAsync(ws.list, 0, sizeof(int) * small_words(g.V, cap), st);
+        }
+      }
+    }
     if constexpr (MIXED) {
       fr_ = VR{reinterpret_cast<typename VR::unit*>(ws.r32), g.V};
       fx_ = VR{reinterpret_cast<typename VR::unit*>(ws.x32), g.V};
@@ -499,7 +526,7 @@ class Engine {
     // The reliable update (FP64, bound by the FP64 pipe) runs on the side
     // stream while the chunk of iterations of the other systems (FP32, bound
     // by memory) runs on the engine's stream: they act on disjoint systems.
-    const bool overlap = ru && run && side_ != nullptr;
+    const bool overlap = ru && run && side_ != nullptr && !small_;
     if (ru) {
       mark_ru<<<(cap_ + 127) / 128, 128, 0, st_>>>(cap_, S);
       launches(1);
@@ -512,7 +539,9 @@ class Engine {
         reliable_update(n_ru, st_, kOver64);
       }
     }
-    if (run) {
+    if (run && small_) {
+      iterate_small();
+    } else if (run) {
       size_for_live();
       // every 4th chunk is timed when profiling, on its second iteration: by
       // then the queue is full, so the events time the kernels rather than the
@@ -578,7 +607,7 @@ class Engine {
   // Whether this engine may run a solve as one device-driven CUDA graph
   // (it needs driver resources, and the kernel-timing samples need the
   // host-driven rounds).
-  bool can_persist() const { return driver_resources_ && side_ != nullptr && !prof(); }
+  bool can_persist() const { return driver_resources_ && side_ != nullptr && !prof() && !small_; }
 
   // Solve the staged systems with one launch of one CUDA graph: the
   // admission kernels, then a conditional WHILE node whose body is one round
@@ -703,7 +732,7 @@ class Engine {
     SysState* S = ws_.S;
     const int gv = grid_of((const void*)admit_clear<VF, NC>, 256, na);
     admit_clear<VF, NC><<<dim3(gv, cap_), 256, 0, st_>>>(g_.V, fp_, vunits_, MIXED ? ws_.x32 : nullptr,
-                                                         MIXED ? n_ : 0, S);
+                                                         MIXED ? runits_ * sizeof(typename VR::unit) / sizeof(float2) : 0, S);
     const int gn = grid_of((const void*)norm_b<NC>, kTile, na);
     if constexpr (MIXED) {
       // b = (D+m)^+ chi in the inner precision: r = p = b and |b|^2
@@ -827,6 +856,41 @@ class Engine {
     launch_k3(g3, ST_JUST_UPDATED, 2, sx, nullptr);
     mark_ready<<<(cap_ + 127) / 128, 128, 0, sx>>>(cap_, S);
     launches(MIXED ? 7 : 5);
+  }
+
+  // Small lattices: many iterations of every running system by one launch (a
+  // launch a window of the list, where the batch exceeds the blocks resident).
+  void iterate_small() {
+    if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
+      constexpr int per = small_traits<OpF>::kPer;
+      const int units = std::max(1, (live_slots() + per - 1) / per), bound = (cap_ + per - 1) / per;
+      // the form with every load under way where each system has blocks of its
+      // own, else the one of which more blocks are resident
+      splan_.wide = small_blocks_[1] >= units * splan_.tiles;
+      splan_.groups = std::max(1, std::min(units, small_blocks_[splan_.wide] / splan_.tiles));
+      splan_.windows = (bound * per + splan_.groups * kSmallShare - 1) / (splan_.groups * kSmallShare);
+      unsigned* bad = reinterpret_cast<unsigned*>(ws_.list + cap_ + 1);
+      build_list<<<1, 256, 0, st_>>>(cap_, ws_.S, ws_.list, bad, splan_.groups, per);
+      for (int w = 0; w < splan_.windows; ++w) {
+        launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
+                     SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epoch_, w,
+                               splan_.windows},
+                     splan_, st_);
+        small_epoch_ += 8 * kSmallIters;
+      }
+      launches(1 + splan_.windows);
+    }
+  }
+
+  // Slots that may run in the next chunk.
+  int live_slots() const {
+    int n = 0;
+    for (int i = 0; i < cap_; ++i) {
+      const int s = hr_[i].status;
+      n += s == ST_RUNNING || s == ST_NEED_RU || s == ST_JUST_UPDATED || s == ST_ADMIT || s == ST_ZERO_GUESS ||
+           s == ST_READY;
+    }
+    return n;
   }
 
   // One graph per grid class (see size_for_live), captured on first use.
@@ -1045,6 +1109,10 @@ class Engine {
                     over);
   }
   int nrun_ = 0, ns_ = 1, gfast_ = 0;
+  bool small_ = false;  // the whole iteration in one cooperative kernel (small.cuh)
+  SmallPlan splan_;
+  int small_blocks_[2] = {0, 0};  // blocks of its two forms resident at once
+  unsigned small_epoch_ = 0;  // barrier epochs used so far
   std::vector<Sample> samples_;
   std::vector<FpSample> fsamples_;
   long long rounds_ = 0, chunks_ = 0;
@@ -1194,7 +1262,8 @@ int run_inner_apply(const Geom& g, const OpF& opf, const double2* in, double2* o
   const size_t vunits = VF::sys_units(g.V), n = (size_t)g.V * NC;
   const int ntiles = (g.V + kTile - 1) / kTile, pstride = kWarps * ntiles;
   const int nsp = pt_systems<VF>(nsys);
-  const size_t bytes = 2 * align_up(sizeof(PU) * vunits * nsp) + align_up(sizeof(float2) * n * nsys) +
+  const size_t rbytes = sizeof(typename VR::unit) * VR::sys_units(g.V) * nsys;
+  const size_t bytes = 2 * align_up(sizeof(PU) * vunits * nsp) + align_up(rbytes) +
                        align_up(sizeof(SysState) * nsys) + align_up(sizeof(double) * pstride * nsys) +
                        align_up(sizeof(unsigned) * nsys);
   DevMem mem;
@@ -1207,7 +1276,7 @@ int run_inner_apply(const Geom& g, const OpF& opf, const double2* in, double2* o
   };
   const VF fp{static_cast<PU*>(take(sizeof(PU) * vunits * nsp)), g.V};
   const VF ft{static_cast<PU*>(take(sizeof(PU) * vunits * nsp)), g.V};
-  const VR fr{static_cast<typename VR::unit*>(take(sizeof(float2) * n * nsys)), g.V};
+  const VR fr{static_cast<typename VR::unit*>(take(rbytes)), g.V};
   const size_t runits = VR::sys_units(g.V);
   SysState* S = static_cast<SysState*>(take(sizeof(SysState) * nsys));
   double* partials = static_cast<double*>(take(sizeof(double) * pstride * nsys));
@@ -1223,7 +1292,7 @@ int run_inner_apply(const Geom& g, const OpF& opf, const double2* in, double2* o
   }
   cudaMemcpyAsync(S, hs.data(), sizeof(SysState) * nsys, cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(tickets, 0, sizeof(unsigned) * nsys, st);
-  cudaMemsetAsync(fr.p, 0, sizeof(float2) * n * nsys, st);
+  cudaMemsetAsync(fr.p, 0, rbytes, st);
   const int gv = grid_for((const void*)demote_chi<NC, VF>, 256, g.V, nsys, ntiles);
   demote_chi<NC, VF><<<dim3(gv, nsys), 256, 0, st>>>(gb, in, dagger ? ft : fp, n, vunits, S);
   set_status<<<(nsys + 127) / 128, 128, 0, st>>>(nsys, S, ST_RUNNING);

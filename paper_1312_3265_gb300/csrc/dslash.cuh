@@ -89,6 +89,25 @@ template <> struct SpLoader<VecP32q<12>, float> {
     return p;
   }
 };
+// FP16: three sixteen-byte loads and the scale
+template <> struct SpLoader<VecP16<12>, float> {
+  static __device__ __forceinline__ Sp<float> load(const VecP16<12>& in, int n) {
+    Sp<float> p;
+    const uint4* b = reinterpret_cast<const uint4*>(in.p) + pk(n, 3, 0);
+    const float s = __ldg(in.sc() + n);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const uint4 v = __ldg(b + q * 16);
+      const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = 4 * q + j;
+        p.s[c / 3].c[c % 3] = s * half2_of(u[j]);
+      }
+    }
+    return p;
+  }
+};
 template <typename In, typename T> __device__ __forceinline__ Sp<T> ld_sp(const In& in, int n) {
   return SpLoader<In, T>::load(in, n);
 }

@@ -48,14 +48,6 @@ template <typename T> __device__ __forceinline__ Sp<T> zero_sp() {
   return a;
 }
 
-// Full index and coordinates of half-lattice site h of parity `par`.
-__device__ __forceinline__ int half_site(const Geom& g, int h, int par, int x[4]) {
-  coords(g, 2 * h, x);
-  const int b = ((x[1] + x[2] + x[3]) & 1) ^ par;  // x0 of site 2h is even
-  x[0] += b;
-  return 2 * h + b;
-}
-
 // acc + sum_mu [(r - c g_mu) U_mu(x) psi(x+mu) + (r + c g_mu) U_mu(x-mu)^+ psi(x-mu)]
 // at full site n; psi is read at the neighbours' half index (HALF) or full
 // index from `in`.  c = -1 for the adjoint.
@@ -225,6 +217,21 @@ __global__ void __launch_bounds__(kTile) eo_prepass(Op op, typename Op::Vec in, 
   const int Vh = op.full.V / 2;
   for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < Vh; h += gridDim.x * blockDim.x)
     op.prepass_site(in, h, (T)op.r, dagger != 0);
+}
+
+// The FP32 Schur operator on small lattices (small.cuh).
+template <typename G, template <int> class VA, bool R1> struct small_traits<WEOOp<float, G, VA, R1>> {
+  static constexpr int kSites = 16, kPer = 1;
+};
+template <typename G, template <int> class VA, bool R1>
+const void* small_kernel(const WEOOp<float, G, VA, R1>&, bool wide) {
+  return wilson_small_kernel<R1, HalfSites, G, VA<12>>(wide);
+}
+template <typename G, template <int> class VA, bool R1>
+void launch_small(const WEOOp<float, G, VA, R1>& op, const GeomBlk&, VA<12> p, VA<12> t, VecP32q<12> r, VecP32q<12> x,
+                  const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
+  launch_cooperative(small_kernel(op, pl.wide), pl, st, HalfSites{op.full}, op.U, p, t, r, x,
+                     op.half_units, a);
 }
 
 // chi^_e = chi_e - D_eo chi_o / M and the even part of the guess, per system,

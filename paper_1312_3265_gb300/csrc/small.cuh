@@ -22,10 +22,18 @@
 // folded into the matrices.
 //
 // Used for lattices whose warps are all resident at once, at most 12 an SM
-// (168 registers a thread); the blocks of a group of systems wait on one
-// another only, and the launch is cooperative, so they are resident together.
+// (168 registers a thread; up to 8 warps and with a group of blocks for every
+// system 255, all hops' loads under way at once); the blocks of a group of
+// systems wait on one another only, and the launch is cooperative, so they are
+// resident together.
 // A wait gives up after kWaitLimit polls: the group's systems are then handed
 // to a reliable update (any x is a valid guess) and the launch ends.
+//
+// An iteration of one system takes 12-14 us, of which the hops are 4, the FP64
+// sums and divisions 3-4 and the fences and inboxes 5.  Measured against the
+// kernels of larger lattices (a solve to 1e-10, same updates): one system, 8^4
+// staggered Wilson 2.87 -> 1.04 ms, 6x10x12x14 Wilson 5.40 -> 2.30; 48 Wilson
+// systems on 8^4 15.0 -> 14.5, on 6x10x12x14 30.7 -> 29.5.
 //
 // The tiles of the reductions depend on the volume only, so a system's
 // results are the same alone and in any batch.
@@ -38,18 +46,26 @@
 namespace swc {
 
 constexpr int kSmallThreads = 384;  // largest block: 12 warps of 168 registers
+constexpr int kSmallWide = 256;     // largest block of the 255-register form
+// Smallest block: fewer warps a block make more blocks that each follow every
+// system of their group (8^4, 48 Wilson systems: 18.7 ms with 2 warps, 16.4
+// with 4, 15.8 with 6, 15.4 with 12), more of them leave one system's sites to
+// few SMs (4^3x8: 1.79, 1.77, 1.79, 2.15 ms).  At least 32 sites a block, for the
+// room of the inboxes.
+constexpr int kSmallWarps = 6;
 constexpr int kSmallShare = 64;     // systems a group of blocks holds
-constexpr int kSmallIters = 32;     // iterations a launch
+constexpr int kSmallIters = 512;    // iterations a launch at most
 constexpr int kWaitLimit = 1 << 22;
 
 // Units (systems, or pairs of them) that run, in order: list[0] = their
 // number, list[1 + i] = (unit << 2) | mask of the unit's systems; systems in
-// ST_READY are set RUNNING first.  Also clears the barrier words.  One block.
-static __global__ void __launch_bounds__(256) build_list(int nsys, SysState* S, int* list, unsigned* bars, int nbars,
+// ST_READY are set RUNNING first.  Also clears the groups' "gave up" words.
+// One block.
+static __global__ void __launch_bounds__(256) build_list(int nsys, SysState* S, int* list, unsigned* bad, int groups,
                                                          int per) {
   __shared__ int wcnt[8];
   const int units = (nsys + per - 1) / per, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < nbars; i += blockDim.x) bars[i] = 0u;
+  for (int i = threadIdx.x; i < groups; i += blockDim.x) bad[i] = 0u;
   int base = 0;
   for (int u0 = 0; u0 < units; u0 += 256) {
     const int u = u0 + threadIdx.x;
@@ -82,95 +98,156 @@ struct SmallArgs {
   RedBuf rb;
   BatchParams bp;
   int nsys;
-  unsigned* bars;  // [groups] arrivals, then [groups] "gave up"
-  int window, windows;  // this launch's part of the list
+  unsigned long long* slots;  // [2][nsys][tiles][tiles][2] each block's inbox: tagged halves of the tile sums
+  unsigned* flags;            // [groups][tiles][tiles] each block's inbox: barrier epochs
+  unsigned* bad;              // [groups] "gave up"
+  unsigned epoch;             // above every epoch of the launches before
+  int window, windows;        // this launch's part of the list
 };
 
-// ---------------------------------------------------------------- the group's state and barrier
+// ---------------------------------------------------------------- the group's state and barriers
 struct SmallShared {
   SysState st[kSmallShare];
   int sys[kSmallShare];  // -1: no system
   int on[kSmallShare];   // still running
   float alpha[kSmallShare], beta[kSmallShare], mass[kSmallShare];
   double wsum[kSmallShare][kSmallThreads / 32];
-  int flag, stopped;
+  int ok;  // no wait has given up
 };
 
-// All blocks of the group (blockIdx.y) have arrived `round` times; false: gave up.
-__device__ __forceinline__ bool group_barrier(const SmallArgs& a, SmallShared& s, unsigned& round) {
-  ++round;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned* c = a.bars + blockIdx.y;
-    unsigned* bad = a.bars + gridDim.y + blockIdx.y;
-    const unsigned want = round * gridDim.x;
-    __threadfence();
-    atomicAdd(c, 1u);
-    int n = 0;
-    unsigned v;
-    s.flag = 1;
-    for (;;) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
-      if (v >= want) break;
-      if (++n > kWaitLimit || ((n & 255) == 0 && atomicAdd(bad, 0u))) {
-        atomicExch(bad, 1u);
-        s.flag = 0;
-        break;
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return s.flag != 0;
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v, unsigned long long w) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(v), "l"(w) : "memory");
+}
+__device__ __forceinline__ void ld_relaxed(const unsigned long long* p, unsigned long long& v, unsigned long long& w) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v), "=l"(w) : "l"(p) : "memory");
+}
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// one more poll in vain: whether to give up
+__device__ __forceinline__ bool give_up(const SmallArgs& a, SmallShared& s, int& n) {
+  if (++n <= kWaitLimit && ((n & 255) || !ld_relaxed(a.bad + blockIdx.y))) return false;
+  atomicExch(a.bad + blockIdx.y, 1u);
+  s.ok = 0;
+  return true;
 }
 
-// The block's sums of this phase -> the tile's slot of buffer `buf`.
-__device__ __forceinline__ void put_tiles(const SmallArgs& a, const SmallShared& s, int share, int buf) {
+constexpr int kPolls = 5;  // tiles a lane polls at once (160 a warp)
+
+// All blocks of the group (blockIdx.y) have reached `epoch`, and their stores
+// before it are visible; false: gave up.
+__device__ __forceinline__ bool group_barrier(const SmallArgs& a, SmallShared& s, unsigned& epoch) {
+  ++epoch;
   __syncthreads();
-  const int nw = blockDim.x >> 5;
-  for (int t = threadIdx.x; t < share; t += blockDim.x) {
+  if (threadIdx.x < 32) {
+    const int nt = gridDim.x;
+    unsigned* f = a.flags + (size_t)blockIdx.y * nt * nt;
+    fence_gpu();
+    for (int i = threadIdx.x; i < nt; i += 32)
+      asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(f + (size_t)i * nt + blockIdx.x), "r"(epoch) : "memory");
+    f += (size_t)blockIdx.x * nt;
+    int n = 0;
+    for (int i0 = threadIdx.x; i0 < nt; i0 += 32 * kPolls) {
+      for (;;) {
+        unsigned v[kPolls];
+#pragma unroll
+        for (int k = 0; k < kPolls; ++k) v[k] = i0 + 32 * k < nt ? ld_relaxed(f + i0 + 32 * k) : epoch;
+        bool all = true;
+#pragma unroll
+        for (int k = 0; k < kPolls; ++k) all &= (int)(v[k] - epoch) >= 0;
+        if (all || give_up(a, s, n)) break;
+      }
+    }
+    __syncwarp();
+    fence_gpu();
+  }
+  __syncthreads();
+  return s.ok != 0;
+}
+
+// A barrier that carries the phase's sums: each block posts its sum of every
+// running system (two 64-bit words, each half of the double tagged with the
+// epoch) into every block's inbox, waits for all tiles' words in its own and
+// adds them in the same order -- one trip through L2 where a counter, its polls
+// and the reading of the sums take three, and no line that all blocks poll
+// (126 blocks polling one array of words held its writers up by 6 us).  Then
+// each block moves its copy of the states on (block 0 records the
+// coefficients).  The slots of a phase are written again only after every block
+// has passed a later barrier.
+template <int PHASE>
+__device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int share, unsigned& epoch) {
+  ++epoch;
+  __syncthreads();
+  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, nt = gridDim.x;
+  const unsigned long long tag = (unsigned long long)epoch << 32;
+  unsigned long long* slots = a.slots + (size_t)(PHASE - 1) * a.nsys * nt * nt * 2;
+  for (int t = threadIdx.x >> 5; t < share; t += nw) {
     if (!s.on[t]) continue;
     double v = s.wsum[t][0];
     for (int w = 1; w < nw; ++w) v += s.wsum[t][w];
-    a.rb.partials[((size_t)buf * a.nsys + s.sys[t]) * a.rb.pstride + blockIdx.x] = v;
+    if (t < nw) fence_gpu();  // the block's stores, before its words
+    const unsigned long long hi = tag | (unsigned)__double2hiint(v), lo = tag | (unsigned)__double2loint(v);
+    for (int i = lane; i < nt; i += 32) st_relaxed(slots + (((size_t)s.sys[t] * nt + i) * nt + blockIdx.x) * 2, hi, lo);
   }
-}
-
-// After the barrier: every block adds the tiles of each running system and
-// moves its copy of the state on (block 0 records the coefficients).
-template <int PHASE> __device__ __forceinline__ void take_tiles(const SmallArgs& a, SmallShared& s, int share, int buf) {
-  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
-  RedBuf rb = a.rb;
-  if (blockIdx.x) rb.hist = nullptr;
+  int n = 0;
   for (int t = threadIdx.x >> 5; t < share; t += nw) {
     if (!s.on[t]) continue;
-    const double* p = a.rb.partials + ((size_t)buf * a.nsys + s.sys[t]) * a.rb.pstride;
+    const unsigned long long* p = slots + ((size_t)s.sys[t] * nt + blockIdx.x) * nt * 2;
     double v = 0.0;
-#pragma unroll 4
-    for (int i = lane; i < (int)gridDim.x; i += 32) v += __ldcg(p + i);
+    for (int i0 = lane; i0 < nt; i0 += 32 * kPolls) {
+      unsigned long long hi[kPolls], lo[kPolls];
+      for (;;) {
+#pragma unroll
+        for (int k = 0; k < kPolls; ++k) {
+          hi[k] = lo[k] = tag;
+          if (i0 + 32 * k < nt) ld_relaxed(p + 2 * (i0 + 32 * k), hi[k], lo[k]);
+        }
+        bool all = true;
+#pragma unroll
+        for (int k = 0; k < kPolls; ++k) all &= (hi[k] >> 32) == epoch && (lo[k] >> 32) == epoch;
+        if (all || give_up(a, s, n)) break;
+      }
+#pragma unroll
+      for (int k = 0; k < kPolls; ++k)
+        if (i0 + 32 * k < nt) v += __hiloint2double((int)(unsigned)hi[k], (int)(unsigned)lo[k]);
+    }
+    __syncwarp();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) {
-      SysState& st = s.st[t];
-      if (PHASE == 1) {
-        finish_k1(st, rb, s.sys[t], v);
-        s.alpha[t] = (float)st.alpha;
-      } else {
-        finish_k2(st, rb, s.sys[t], v);
-        s.beta[t] = (float)st.beta;
-      }
-      if (st.status != ST_RUNNING) s.on[t] = 0;
+    if (lane == 0) s.wsum[t][0] = v;
+  }
+  fence_gpu();
+  __syncthreads();
+  // one thread a system: the divisions of all systems at once
+  RedBuf rb = a.rb;
+  if (blockIdx.x) rb.hist = nullptr;
+  for (int t = threadIdx.x; t < share; t += blockDim.x) {
+    if (!s.on[t]) continue;
+    SysState& st = s.st[t];
+    if (PHASE == 1) {
+      finish_k1(st, rb, s.sys[t], s.wsum[t][0]);
+      s.alpha[t] = (float)st.alpha;
+    } else {
+      finish_k2(st, rb, s.sys[t], s.wsum[t][0]);
+      s.beta[t] = (float)st.beta;
     }
+    if (st.status != ST_RUNNING) s.on[t] = 0;
   }
   __syncthreads();
+  return s.ok != 0;
 }
 
 // The group's part of the list -> shared memory; returns its size (systems).
 __device__ __forceinline__ int load_share(const SmallArgs& a, SmallShared& s, int per) {
+  // every parts-th unit: neighbours in the batch often stop together (one mass),
+  // and a group whose systems stop at different iterations keeps its SMs busy
   const int cnt = a.list[0], parts = a.windows * gridDim.y, part = a.window * gridDim.y + blockIdx.y;
-  const int lo = (int)((long long)cnt * part / parts), n = (int)((long long)cnt * (part + 1) / parts) - lo;
+  const int n = part < cnt ? (cnt - part - 1) / parts + 1 : 0;
   for (int t = threadIdx.x; t < n * per; t += blockDim.x) {
-    const int e = a.list[1 + lo + t / per], sys = (e >> 2) * per + t % per;
+    const int e = a.list[1 + part + (t / per) * parts], sys = (e >> 2) * per + t % per;
     const bool run = (e >> (t % per)) & 1;
     s.sys[t] = run ? sys : -1;
     s.on[t] = run;
@@ -180,7 +257,7 @@ __device__ __forceinline__ int load_share(const SmallArgs& a, SmallShared& s, in
       s.mass[t] = (float)s.st[t].mass;
     }
   }
-  if (threadIdx.x == 0) s.stopped = 0;
+  if (threadIdx.x == 0) s.ok = 1;
   __syncthreads();
   return n * per;
 }
@@ -198,7 +275,10 @@ __device__ __forceinline__ bool group_goes_on(const SmallShared& s, int share) {
 
 __device__ __forceinline__ void store_states(const SmallArgs& a, const SmallShared& s, int share, bool gave_up) {
   __syncthreads();
-  if (blockIdx.x && !gave_up) return;
+  if (!gave_up) {
+    if (blockIdx.x) return;
+    gave_up = ld_relaxed(a.bad + blockIdx.y) != 0;  // another block did, at the last barrier
+  }
   for (int t = threadIdx.x; t < share; t += blockDim.x) {
     if (s.sys[t] < 0) continue;
     if (gave_up) {  // (every block writes the same)
@@ -212,19 +292,43 @@ __device__ __forceinline__ void store_states(const SmallArgs& a, const SmallShar
   }
 }
 
-// A warp's FP32 norms (NV values a system) of up to 8 systems, added in FP64
-// by 4 lanes a system: few instructions of the FP64 pipe.
+// The FP64 sum of a warp's FP32 norms (NV lanes a system), lane l with l ^ 1,
+// then ^ 2, ^ 4, ...  For up to 8 systems at once 4 lanes a system add NV / 4
+// values each (the FP64 pipe takes 64 clocks a warp's instruction: 17 of them
+// for 8 systems, or 5 a system by the tree of shuffles, which is therefore
+// taken for one or two systems).  Both add in the same order.
 template <int NV> struct NormBuf { float v[8][NV + 1]; };
 template <int NV>
 __device__ __forceinline__ void flush_norms(NormBuf<NV>& b, SmallShared& sh, int slot0, int nslot) {
-  const int lane = threadIdx.x & 31, s = lane >> 2, q = lane & 3;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __syncwarp();
-  double a = 0.0;
+  if (nslot <= 2) {
+    if (NV == 32 || nslot == 1) {
+      for (int s = 0; s < nslot; ++s) {
+        double a = (double)b.v[s][lane % NV];
 #pragma unroll
-  for (int j = 0; j < NV / 4; ++j) a += (double)b.v[s][q * (NV / 4) + j];
-  a += __shfl_xor_sync(0xffffffffu, a, 1);
-  a += __shfl_xor_sync(0xffffffffu, a, 2);
-  if (q == 0 && s < nslot) sh.wsum[slot0 + s][threadIdx.x >> 5] = a;
+        for (int o = 1; o < NV; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) sh.wsum[slot0 + s][warp] = a;
+      }
+    } else {  // two systems, 16 lanes each
+      double a = (double)b.v[lane / NV][lane % NV];
+#pragma unroll
+      for (int o = 1; o < NV; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane % NV == 0) sh.wsum[slot0 + lane / NV][warp] = a;
+    }
+  } else {
+    const int s = lane >> 2, q = lane & 3;
+    double a[NV / 4];
+#pragma unroll
+    for (int j = 0; j < NV / 4; ++j) a[j] = (double)b.v[s][q * (NV / 4) + j];
+#pragma unroll
+    for (int o = 1; o < NV / 4; o <<= 1)
+#pragma unroll
+      for (int j = 0; j < NV / 4; j += 2 * o) a[j] += a[j + o];
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+    if (q == 0 && s < nslot) sh.wsum[slot0 + s][warp] = a[0];
+  }
   __syncwarp();
 }
 
@@ -267,11 +371,6 @@ template <> struct SpinorIO<VecP32q<12>> {
     for (int k = 0; k < 3; ++k) b[k * 16] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
   }
 };
-__device__ __forceinline__ cx<float> half2_of(unsigned u) {
-  __half2 h;
-  memcpy(&h, &u, 4);
-  return h2c(h);
-}
 template <> struct SpinorIO<VecP16<12>> {
   struct Raw { uint4 q[3]; float s; };
   __device__ static __forceinline__ unsigned offset(int n) { return (unsigned)pk(n, 3, 0); }
@@ -372,8 +471,8 @@ struct HalfSites {
 };
 
 // scratch: units from a system's vector to its scratch (even-odd operator)
-template <bool R1, class Sites, class GA, class VI>
-__global__ void __launch_bounds__(kSmallThreads, 1)
+template <int MAXT, bool R1, class Sites, class GA, class VI>
+__global__ void __launch_bounds__(MAXT, 1)
     wilson_small(Sites sites, GA U, VI p, VI t, VecP32q<12> r, VecP32q<12> x, size_t scratch, SmallArgs a) {
   using IO = SpinorIO<VI>;
   using RO = SpinorIO<VecP32q<12>>;
@@ -414,11 +513,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     Sp<float> acc;
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc.s[k] = zero3<float>();
-    typename IO::Raw raw = IO::load(in, off[0], vi[0]);
+    constexpr int kAhead = MAXT <= kSmallWide ? 4 : 1;  // hops whose loads are under way: all of them where registers allow
+    typename IO::Raw raw[4];
+#pragma unroll
+    for (int mu = 0; mu < kAhead; ++mu) raw[mu] = IO::load(in, off[mu], vi[mu]);
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-      const Sp<float> q = IO::unpack(raw);
-      if (mu < 3) raw = IO::load(in, off[mu + 1], vi[mu + 1]);  // one hop ahead of the arithmetic
+      const Sp<float> q = IO::unpack(raw[mu]);
+      if (mu + kAhead < 4) raw[mu + kAhead] = IO::load(in, off[mu + kAhead], vi[mu + kAhead]);
       if constexpr (R1) {
         V3<float> h0, h1;
         wproject(mu, sg, q, h0, h1);
@@ -443,7 +545,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     v.p += scratch;
     return v;
   };
-  unsigned round = 0;
+  unsigned epoch = a.epoch;
   // even-odd: u = D_oe v of every running system into v's scratch
   auto odd_pass = [&](const VI& v, bool dagger) {
     load_links(1);
@@ -456,7 +558,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       for (int c = 0; c < 12; ++c) o[c] *= -0.5f;
       IO::store_half(aside(w), n, half, on, o);
     }
-    if (!group_barrier(a, s, round)) return false;
+    if (!group_barrier(a, s, epoch)) return false;
     load_links(0);
     return true;
   };
@@ -484,9 +586,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       }
       if ((k & 7) == 7 || k == share - 1) flush_norms<32>(nbuf[warp], s, k & ~7, (k & 7) + 1);
     }
-    put_tiles(a, s, share, 0);
-    if (!(ok = group_barrier(a, s, round))) break;
-    take_tiles<1>(a, s, share, 0);
+    if (!(ok = exchange<1>(a, s, share, epoch))) break;
     if constexpr (kEO)
       if (!(ok = odd_pass(t, true))) break;
 #pragma unroll 1
@@ -510,9 +610,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       }
       if ((k & 7) == 7 || k == share - 1) flush_norms<32>(nbuf[warp], s, k & ~7, (k & 7) + 1);
     }
-    put_tiles(a, s, share, 1);
-    if (!(ok = group_barrier(a, s, round))) break;
-    take_tiles<2>(a, s, share, 1);
+    if (!(ok = exchange<2>(a, s, share, epoch))) break;
     const bool more = group_goes_on(s, share);
 #pragma unroll 1
     for (int k = 0; k < share; ++k) {
@@ -533,7 +631,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       IO::store_half(w, n, half, on, pv);
     }
     if (!more) break;
-    if (!(ok = group_barrier(a, s, round))) break;
+    if (!(ok = group_barrier(a, s, epoch))) break;
   }
   store_states(a, s, share, !ok);
 }
@@ -630,8 +728,8 @@ __device__ __forceinline__ M3<float> scaled(float c, const M3<float>& A) {
   return B;
 }
 
-template <class GG, class GA, class TA, class VI>
-__global__ void __launch_bounds__(kSmallThreads, 1)
+template <int MAXT, class GG, class GA, class TA, class VI>
+__global__ void __launch_bounds__(MAXT, 1)
     sw_small(GG g, GA U, TA W, VI p, VI t, VecP32<3> r, VecP32<3> x, SmallArgs a) {
   using IO = PairIO<VI>;
   __shared__ SmallShared s;
@@ -674,10 +772,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   // this lane's 3 numbers of sum of the hops and corners
   auto hops = [&](const typename IO::View& in, float o[3]) {
     V3<float> acc[2] = {zero3<float>(), zero3<float>()};
+    typename IO::Raw raw[6];
+#pragma unroll
+    for (int h = 0; h < 6; ++h) raw[h] = IO::load(in, off[h]);
 #pragma unroll
     for (int h = 0; h < 6; ++h) {
       V3<float> v[2];
-      IO::unpack(IO::load(in, off[h]), v);
+      IO::unpack(raw[h], v);
       mv_acc(acc[0], M[h], v[0]);
       mv_acc(acc[1], M[h], v[1]);
     }
@@ -704,7 +805,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   auto rpart = [&](const VecP32<3>& v, int s0) {
     return reinterpret_cast<float*>(v.p + (size_t)(s0 + ls) * a.bp.sstride + pk(n, 3, 0)) + part;
   };
-  unsigned round = 0;
+  unsigned epoch = a.epoch;
   bool ok = true;
   for (int it = 0; it < kSmallIters; ++it) {
 #pragma unroll 1
@@ -724,9 +825,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       }
       if ((k & 7) == 6 || k == share - 2) flush_norms<16>(nbuf[warp], s, k & ~7, (k & 7) + 2);
     }
-    put_tiles(a, s, share, 0);
-    if (!(ok = group_barrier(a, s, round))) break;
-    take_tiles<1>(a, s, share, 0);
+    if (!(ok = exchange<1>(a, s, share, epoch))) break;
     adjoint();
 #pragma unroll 1
     for (int k = 0; k < share; k += 2) {
@@ -755,9 +854,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       if ((k & 7) == 6 || k == share - 2) flush_norms<16>(nbuf[warp], s, k & ~7, (k & 7) + 2);
     }
     adjoint();
-    put_tiles(a, s, share, 1);
-    if (!(ok = group_barrier(a, s, round))) break;
-    take_tiles<2>(a, s, share, 1);
+    if (!(ok = exchange<2>(a, s, share, epoch))) break;
     const bool more = group_goes_on(s, share);
 #pragma unroll 1
     for (int k = 0; k < share; k += 2) {
@@ -781,7 +878,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       IO::store_part(IO::view(p, s0, 3, a.bp.vstride), n, ls, part, on && st, pv);
     }
     if (!more) break;
-    if (!(ok = group_barrier(a, s, round))) break;
+    if (!(ok = group_barrier(a, s, epoch))) break;
   }
   store_states(a, s, share, !ok);
 }
@@ -798,47 +895,64 @@ template <typename G, template <int> class VA, bool R1, bool LEAN> struct small_
 
 struct SmallPlan {
   int nt = 0, tiles = 0, groups = 1, windows = 1;
+  bool wide = false;
 };
+
+// Tiles a small lattice can have (0: too large for any operator), for the
+// workspace: its blocks hold at least 32 sites and are at most one per SM.
+inline size_t small_tiles_bound(int V) {
+  return V > sm_count() * kSmallThreads / 2 ? 0 : std::min<size_t>(sm_count(), ((size_t)V + 31) / 32);
+}
+inline size_t small_slots(int V, int nsys) {  // 64-bit words of the inboxes
+  return 4 * small_tiles_bound(V) * small_tiles_bound(V) * nsys;
+}
+inline size_t small_words(int V, int nsys) {  // ints: list, "gave up" words, barrier epochs
+  return small_tiles_bound(V) ? 1 + 2 * (size_t)nsys + small_tiles_bound(V) * small_tiles_bound(V) * nsys : 0;
+}
 
 // Whether a lattice of V sites (of the operator's vectors) takes the small
 // form, and its blocks: as few warps a block as spread the lattice over every
-// SM (at least 32 sites a block, the room of the reduction's slots).  By the
-// volume only.
+// SM.  By the volume only.
 inline bool small_tiles(int V, int sites_per_warp, SmallPlan* p) {
   const int sms = sm_count();
   const long long warps = (V + sites_per_warp - 1) / sites_per_warp;
   if (warps > (long long)sms * (kSmallThreads / 32)) return false;
   int per = (int)((warps + sms - 1) / sms);
-  per = std::max(per, 32 / sites_per_warp);
+  per = std::max(per, kSmallWarps);
   p->nt = 32 * per;
   p->tiles = (int)((warps + per - 1) / per);
   return true;
 }
 
-template <class Kernel, class... Args>
-void launch_cooperative(Kernel k, const SmallPlan& p, cudaStream_t st, Args... args) {
+template <class... Args>
+void launch_cooperative(const void* kernel, const SmallPlan& p, cudaStream_t st, Args... args) {
   void* v[] = {(void*)&args...};
-  cudaLaunchCooperativeKernel((const void*)k, dim3(p.tiles, p.groups), dim3(p.nt), v, 0, st);
+  cudaLaunchCooperativeKernel(kernel, dim3(p.tiles, p.groups), dim3(p.nt), v, 0, st);
 }
 
+// the kernel of an operator (wide: the 255-register form), and its launch
 template <typename G, typename Wt, template <int> class VA>
-const void* small_kernel(const SWOp<float, G, Wt, VA>&) {
-  return (const void*)sw_small<GeomBlk, G, Wt, VA<3>>;
+const void* small_kernel(const SWOp<float, G, Wt, VA>&, bool wide) {
+  return wide ? (const void*)sw_small<kSmallWide, GeomBlk, G, Wt, VA<3>>
+              : (const void*)sw_small<kSmallThreads, GeomBlk, G, Wt, VA<3>>;
 }
 template <typename G, typename Wt, template <int> class VA>
 void launch_small(const SWOp<float, G, Wt, VA>& op, const GeomBlk& g, VA<3> p, VA<3> t, VecP32<3> r, VecP32<3> x,
                   const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
-  launch_cooperative(sw_small<GeomBlk, G, Wt, VA<3>>, pl, st, g, op.U, op.W, p, t, r, x, a);
+  launch_cooperative(small_kernel(op, pl.wide), pl, st, g, op.U, op.W, p, t, r, x, a);
+}
+template <bool R1, class Sites, class GA, class VI> const void* wilson_small_kernel(bool wide) {
+  return wide ? (const void*)wilson_small<kSmallWide, R1, Sites, GA, VI>
+              : (const void*)wilson_small<kSmallThreads, R1, Sites, GA, VI>;
 }
 template <typename G, template <int> class VA, bool R1, bool LEAN>
-const void* small_kernel(const WOp<float, G, VA, R1, LEAN>&) {
-  return (const void*)wilson_small<R1, FullSites<GeomBlk>, G, VA<12>>;
+const void* small_kernel(const WOp<float, G, VA, R1, LEAN>&, bool wide) {
+  return wilson_small_kernel<R1, FullSites<GeomBlk>, G, VA<12>>(wide);
 }
 template <typename G, template <int> class VA, bool R1, bool LEAN>
 void launch_small(const WOp<float, G, VA, R1, LEAN>& op, const GeomBlk& g, VA<12> p, VA<12> t, VecP32q<12> r,
                   VecP32q<12> x, const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
-  launch_cooperative(wilson_small<R1, FullSites<GeomBlk>, G, VA<12>>, pl, st, FullSites<GeomBlk>{g}, op.U, p, t, r, x,
-                     size_t(0), a);
+  launch_cooperative(small_kernel(op, pl.wide), pl, st, FullSites<GeomBlk>{g}, op.U, p, t, r, x, size_t(0), a);
 }
 
 }  // namespace swc
