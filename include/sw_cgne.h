@@ -213,8 +213,10 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  * SW_PARAM_RELIABLE_DELTA: mixed precision only; the FP32 correction is
  *   folded into the FP64 solution and r = b - A x recomputed in FP64 when the
  *   iterated |r| falls below delta times its maximum since the last such
- *   update (Sleijpen & van der Vorst 1996); (0, 1), default 3e-5.  Applies to
- *   SW_PREC_F32_RELIABLE.
+ *   update (Sleijpen & van der Vorst 1996); (0, 1), default 3e-5.  A solve is
+ *   cut into the fewest equal legs that reduce the residual by about delta
+ *   each (tol 1e-8: 2 of 1e-4; 1e-10: 2 of 1e-5; 1e-12: 3 of 1e-4).  Applies
+ *   to SW_PREC_F32_RELIABLE.
  * SW_PARAM_RELIABLE_DELTA_F16: the same trigger for SW_PREC_F16_RELIABLE,
  *   default 1e-3: FP16 storage drifts from the true residual about four
  *   orders of magnitude sooner than FP32, and CG loses its conjugacy if the

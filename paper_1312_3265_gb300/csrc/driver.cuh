@@ -18,6 +18,7 @@
 #pragma once
 #include <algorithm>
 #include <chrono>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -172,6 +173,18 @@ inline double* pinned_hist(size_t n) {
     cap = n;
   }
   return buf;
+}
+
+// Reliable-update trigger of a system from its tolerance: the solve is cut into
+// the fewest legs that reduce the residual by about `delta` each, and the legs
+// are made equal, delta = tol^(1/legs) -- a trigger of delta itself leaves a
+// short last leg, whose FP64 residual costs as much as the others'.  A leg may
+// go a quarter (in the logarithm) below delta where that saves one: at 3e-5
+// FP32 iterations keep their count down to 1e-5.  tol 1e-8: 2 legs of 1e-4;
+// 1e-10: 2 of 1e-5 (by 3e-5: 3); 1e-12: 3 of 1e-4.
+inline double leg_delta(double tol, double delta) {
+  const double legs = std::max(1.0, std::ceil(std::log(tol) / std::log(delta) - 0.25));
+  return std::pow(tol, 1.0 / legs);
 }
 
 inline int status_to_code(int st) {
@@ -493,7 +506,8 @@ class Engine {
     SysState s{};
     s.tol2 = tol * tol;
     s.cb2 = cb2;
-    s.delta2 = MIXED ? delta_ * delta_ : 0.0;
+    const double leg = MIXED ? leg_delta(tol, delta_) : 0.0;
+    s.delta2 = leg * leg;
     s.max_iter = max_iter;
     s.mass = mass;
     s.status = ST_ADMIT;
