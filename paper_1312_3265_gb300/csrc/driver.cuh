@@ -65,6 +65,15 @@ template <class Op> bool use_quad(int V) {
   return false;
 }
 constexpr int kOver64 = 8;  // waves of blocks of the FP64 kernels
+// A chunk runs as two halves (Engine::run_chunk) from this many complex numbers in
+// a vector of the running systems (below, a half's launches are as short as the
+// host takes to issue them), where the stored gauge data of the operator take at
+// most kSplitGauge bytes: both halves read them from L2.  A solve to 1e-10, whole
+// against halves, ms: Wilson FP32 12^3x24, 12 systems 29.0 / 25.5; 16^3x32, 48:
+// 256 / 237; FP16 12^3x24 38.9 / 33.9; even-odd 16^3x32, 12: 42.2 / 39.8;
+// staggered Wilson 16^4, 12 (57 MB): 17.0 / 15.6 -- but 16^3x32, 24 (113 MB): 52.3
+// / 54.0 and 24^3x48, 24 (573 MB): 252 / 258; Wilson 24^3x48 (191 MB) 358 / 356.
+constexpr double kSplitWork = 1 << 21, kSplitGauge = 80e6;
 
 // over: waves of blocks at most.  Kernels bound by the FP64 pipe take several:
 // blocks that share the pipe do not run in rounds, and a block that loops over
@@ -338,7 +347,7 @@ class Engine {
          const Workspace& ws, SysState* hs_read, SysState* hs_stage, cudaStream_t st, cudaEvent_t ev,
          bool use_graphs = true)
       : g_(g), opd_(opd), opf_(opf), r_(r), cap_(cap), chi_(chi), x_(x), ws_(ws), hr_(hs_read), hst_(hs_stage),
-        st_(st), ist_(st), ev_(ev), n_((size_t)g.V * NC), s64_(n_ * f64_stride_factor<OpD>()),
+        st_(st), ev_(ev), n_((size_t)g.V * NC), s64_(n_ * f64_stride_factor<OpD>()),
         use_graphs_(use_graphs && param_graphs()),
         driver_resources_(use_graphs) {
     ntiles_ = (g.V + kTile - 1) / kTile;
@@ -357,7 +366,14 @@ class Engine {
     bp_ = BatchParams{r, runits_, s64_, vunits_};
     ns_ = MIXED ? param_ns(NC) : 1;
     ngrp_ = (cap + ns_ - 1) / ns_;
-    set_grids(ngrp_);
+    whole_.n = cap;
+    whole_.ngrp = ngrp_;
+    // halves of whole groups (and pairs)
+    half_[0].n = half_[1].s0 = (ngrp_ + 1) / 2 * ns_ & ~1;
+    half_[1].n = cap - half_[0].n;
+    for (Range& h : half_) h.ngrp = (h.n + ns_ - 1) / ns_;
+    cls_ = ngrp_;
+    set_grids(whole_, ngrp_);
     if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
       small_ = small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
       if (small_) {
@@ -401,6 +417,13 @@ class Engine {
           cudaEventCreateWithFlags(&ev_join_, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         side_ = nullptr;
+      }
+      if (MIXED && !small_ && cap_ >= 2 * std::max(2, ns_) &&
+          (cudaStreamCreateWithFlags(&half_st_, cudaStreamNonBlocking) != cudaSuccess ||
+           cudaEventCreateWithFlags(&ev_split_, cudaEventDisableTiming) != cudaSuccess ||
+           cudaEventCreateWithFlags(&ev_meet_, cudaEventDisableTiming) != cudaSuccess)) {
+        cudaGetLastError();
+        half_st_ = nullptr;
       }
     }
     cudaMemsetAsync(ws.pcount, 0, sizeof(int) * 2 * kProfSlots, st);
@@ -484,6 +507,12 @@ class Engine {
       cudaStreamSynchronize(side_);
       cudaStreamDestroy(side_);
     }
+    if (half_st_) {
+      cudaStreamSynchronize(half_st_);
+      cudaStreamDestroy(half_st_);
+    }
+    if (ev_split_) cudaEventDestroy(ev_split_);
+    if (ev_meet_) cudaEventDestroy(ev_meet_);
     if (ev_fork_) cudaEventDestroy(ev_fork_);
     if (ev_join_) cudaEventDestroy(ev_join_);
   }
@@ -568,7 +597,7 @@ class Engine {
       if (!prof && use_graphs_ && chunks_ > 1) {
         launch_chunk_graph();
       } else {
-        for (int i = 0; i < chunk_; ++i) iterate(prof && i == 1);
+        run_chunk(prof, true);
       }
     }
     if (overlap) cudaStreamWaitEvent(st_, ev_join_, 0);
@@ -642,7 +671,8 @@ class Engine {
     if (staged_.empty()) return 0;
     const int na = (int)staged_.size();
     upload_staged();
-    set_grids(ngrp_);
+    cls_ = ngrp_;
+    set_grids(whole_, ngrp_);
     SysState* S = ws_.S;
     cudaMemsetAsync(ws_.ctl, 0, sizeof(int) * 8, st_);
     cudaStream_t body_st = nullptr;
@@ -675,19 +705,18 @@ class Engine {
         ok = cudaStreamBeginCaptureToGraph(body_st, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
-          ist_ = body_st;
           mark_ru<<<(cap_ + 127) / 128, 128, 0, body_st>>>(cap_, S);
           cudaEventRecord(ev_fork_, body_st);
           cudaStreamWaitEvent(side_, ev_fork_, 0);
           reliable_update(cap_, side_);
           cudaEventRecord(ev_join_, side_);
-          for (int i = 0; i < chunk_; ++i) iterate(false, false);
+          commit(whole_, body_st);
+          for (int i = 0; i < chunk_; ++i) iterate(whole_, body_st, false, false);
           cudaStreamWaitEvent(body_st, ev_join_, 0);
           round_end<<<1, 256, 0, body_st>>>(cap_, S, ws_.ctl, max_rounds, loop);
-          ist_ = st_;
           cudaGraph_t body = nullptr;
           ok = cudaStreamEndCapture(body_st, &body) == cudaSuccess;
-          per_round = 2 + (MIXED ? 7 : 5) + 4 * chunk_ + (two_pass<OpF>::value ? 2 * chunk_ + 2 : 0);
+          per_round = 3 + (MIXED ? 7 : 5) + 3 * chunk_ + (two_pass<OpF>::value ? 2 * chunk_ + 2 : 0);
         }
       }
       ok = ok && cudaStreamUpdateCaptureDependencies(st_, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies) ==
@@ -701,7 +730,6 @@ class Engine {
     capturing_ = false;
     if (graph) cudaGraphDestroy(graph);
     if (body_st) cudaStreamDestroy(body_st);
-    ist_ = st_;
     if (!ok) {
       if (exec) cudaGraphExecDestroy(exec);
       cudaGetLastError();
@@ -733,9 +761,10 @@ class Engine {
   // intermediate field of `in`'s systems in `status`, before the operator
   // is applied to them.
   template <class Op, class Vec>
-  void prepass(const Op& op, const Vec& in, size_t stride, int status, bool dagger, cudaStream_t s) {
+  void prepass(const Op& op, const Vec& in, size_t stride, int status, bool dagger, cudaStream_t s, int s0 = 0,
+               int n = -1) {
     if constexpr (two_pass<Op>::value) {
-      op.prepass(in, stride, ws_.S, status, dagger ? 1 : 0, cap_, s);
+      op.prepass(in, stride, ws_.S + s0, status, dagger ? 1 : 0, n < 0 ? cap_ : n, s);
       launches(1);
     }
   }
@@ -916,7 +945,7 @@ class Engine {
       cudaGraph_t graph = nullptr;
       bool ok = cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
       if (ok) {
-        for (int i = 0; i < chunk_; ++i) iterate(false, false);
+        run_chunk(false, false);
         ok = cudaStreamEndCapture(st_, &graph) == cudaSuccess && graph;
       }
       ok = ok && cudaGraphInstantiate(&ge, graph, 0) == cudaSuccess;
@@ -931,52 +960,104 @@ class Engine {
     }
     if (ge) {
       cudaGraphLaunch(ge, st_);
-      launches(4 * chunk_);
+      launches((split_ ? 2 : 1) * (1 + 3 * chunk_));
       if (prof()) {
         prof_count(cls_k1(), chunk_);
         prof_count(cls_k2(), chunk_);
         prof_count(cls_k3(), chunk_);
       }
     } else {
-      for (int i = 0; i < chunk_; ++i) iterate(false);
+      run_chunk(false, true);
     }
   }
 
-  // Grids of the iteration kernels for `groups` groups of ns_ slots that may
-  // run (blocks of stopped slots return at once).
-  void set_grids(int groups) {
-    cls_ = groups;
+  // Consecutive slots whose iterations are launched together, and their grids.
+  struct Range {
+    int s0 = 0, n = 0, ngrp = 0, g1 = 0, g2 = 0, gV = 0;
+  };
+
+  // READY -> RUNNING, at a chunk's start.
+  void commit(const Range& q, cudaStream_t s) { commit_ready<<<(q.n + 127) / 128, 128, 0, s>>>(q.n, ws_.S + q.s0); }
+
+  // A chunk of iterations on the engine's stream -- or as two halves of the
+  // slots on two streams, which share nothing but the gauge field: one half's
+  // streaming k3 (bound by memory) and the tails of its launches then run
+  // beside the other's stencils (bound by the loads in flight).
+  void run_chunk(bool sample, bool count) {
+    if (split_) {
+      cudaEventRecord(ev_split_, st_);
+      cudaStreamWaitEvent(half_st_, ev_split_, 0);
+      commit(half_[0], st_);
+      commit(half_[1], half_st_);
+      for (int i = 0; i < chunk_; ++i) {
+        iterate(half_[0], st_, false, count);
+        iterate(half_[1], half_st_, false, count);
+      }
+      cudaEventRecord(ev_meet_, half_st_);
+      cudaStreamWaitEvent(st_, ev_meet_, 0);
+      if (count) launches(2);
+    } else {
+      commit(whole_, st_);
+      for (int i = 0; i < chunk_; ++i) iterate(whole_, st_, sample && i == 1, count);
+      if (count) launches(1);
+    }
+  }
+
+  // Grids of the iteration kernels of a range for `groups` groups of ns_ slots
+  // that may run (blocks of stopped slots return at once).
+  void set_grids(Range& q, int groups) {
     if (MIXED || !use_quad<OpF>(g_.V)) {
       if constexpr (MIXED || !quad_always<OpF>()) {
-        g1_ = grid_for(k1_ptr(), kTile, g_.V, groups, ntiles_, MIXED ? 1 : kOver64);
-        g2_ = grid_for(k2_ptr(), kTile, g_.V, groups, ntiles_, MIXED ? 1 : kOver64);
+        q.g1 = grid_for(k1_ptr(), kTile, g_.V, groups, ntiles_, MIXED ? 1 : kOver64);
+        q.g2 = grid_for(k2_ptr(), kTile, g_.V, groups, ntiles_, MIXED ? 1 : kOver64);
       }
     } else if constexpr (!MIXED && has_quad<OpF>()) {
-      g1_ = grid_for((const void*)iter_quad<1, OpF>, kTile, 4LL * g_.V, groups, ntiles_ * 4, kOver64);
-      g2_ = grid_for((const void*)iter_quad<2, OpF>, kTile, 4LL * g_.V, groups, ntiles_ * 4, kOver64);
+      q.g1 = grid_for((const void*)iter_quad<1, OpF>, kTile, 4LL * g_.V, groups, ntiles_ * 4, kOver64);
+      q.g2 = grid_for((const void*)iter_quad<2, OpF>, kTile, 4LL * g_.V, groups, ntiles_ * 4, kOver64);
     }
-    gV_ = grid_for(k3_ptr(), 256, g_.V, k3_rows(groups * ns_), ntiles_);
+    q.gV = grid_for(k3_ptr(), 256, g_.V, k3_rows(groups * ns_), ntiles_);
   }
 
-  // Size the iteration grids for the groups holding a slot that may run in
-  // the next chunk, rounded up to a power of two (at most the engine's
-  // groups): as systems converge, the remaining ones keep the SMs full.  A
-  // system's arithmetic and reduction order do not depend on the grid.
-  void size_for_live() {
+  // Groups of a range holding a slot that may run in the next chunk, rounded up
+  // to a power of two (at most the range's groups): as systems converge, the
+  // remaining ones keep the SMs full.  A system's arithmetic and reduction order
+  // do not depend on the grid.
+  int live_class(const Range& q, int* systems) const {
     int live = 0;
-    for (int gi = 0; gi < ngrp_; ++gi) {
+    for (int gi = 0; gi < q.ngrp; ++gi) {
       bool any = false;
-      for (int i = gi * ns_; i < cap_ && i < (gi + 1) * ns_; ++i) {
+      for (int i = q.s0 + gi * ns_; i < q.s0 + q.n && i < q.s0 + (gi + 1) * ns_; ++i) {
         const int s = hr_[i].status;
-        any |= (s == ST_RUNNING || s == ST_NEED_RU || s == ST_JUST_UPDATED || s == ST_ADMIT || s == ST_ZERO_GUESS ||
-                s == ST_READY);
+        const bool on = s == ST_RUNNING || s == ST_NEED_RU || s == ST_JUST_UPDATED || s == ST_ADMIT ||
+                        s == ST_ZERO_GUESS || s == ST_READY;
+        any |= on;
+        *systems += on;
       }
       live += any;
     }
     int cls = 1;
     while (cls < live) cls *= 2;
-    if (cls > ngrp_) cls = ngrp_;
-    if (cls != cls_) set_grids(cls);
+    return live ? std::min(cls, q.ngrp) : 0;
+  }
+
+  // Size the iteration grids for the slots that may run in the next chunk, and
+  // decide whether it runs as two halves: with systems in both, and enough of
+  // them that a half's launches are longer than the host takes to issue two.
+  void size_for_live() {
+    int n0 = 0, n1 = 0;
+    const bool may = half_st_ && !prof() && (double)g_.V * OpF::kGaugeBytes <= kSplitGauge;
+    const int a = may ? live_class(half_[0], &n0) : 0, b = a ? live_class(half_[1], &n1) : 0;
+    split_ = a && b && (double)g_.V * NC * (n0 + n1) >= kSplitWork;
+    int n = 0;
+    const long long cls = split_ ? ((long long)a << 32) + b : std::max(1, live_class(whole_, &n));
+    if (cls == cls_) return;
+    cls_ = cls;
+    if (split_) {
+      set_grids(half_[0], a);
+      set_grids(half_[1], b);
+    } else {
+      set_grids(whole_, (int)cls);
+    }
   }
 
   void flush_fp_samples() {
@@ -1013,50 +1094,63 @@ class Engine {
     }
     return (const void*)cg_k2<TF, OpF, 1, VR, GK>;
   }
-  template <int NS> void launch_k12(int* c) {
-    SysState* S = ws_.S;
-    const dim3 grid1 = gfast_ ? dim3(ngrp_, g1_) : dim3(g1_, ngrp_), grid2 = gfast_ ? dim3(ngrp_, g2_) : dim3(g2_, ngrp_);
-    prepass(opf_, fp_, vunits_, ST_RUNNING, false, ist_);
-    cg_k1<TF, OpF, NS, GK><<<grid1, kTile, 0, ist_>>>(gk_, opf_, fp_, ft_, bp_, cap_, S, rb_, c, gfast_);
-    if (c) cudaEventRecord(samples_.back().e1, ist_);
-    prepass(opf_, ft_, vunits_, ST_RUNNING, true, ist_);
-    cg_k2<TF, OpF, NS, VR, GK><<<grid2, kTile, 0, ist_>>>(gk_, opf_, ft_, fr_, bp_, cap_, S, rb_,
-                                                          c ? c + 1 : nullptr, gfast_);
+  // A range's view of the batch: vectors, states, reduction buffers.
+  template <class V> static V shifted(V v, size_t units) {
+    v.p += units;
+    return v;
+  }
+  RedBuf shifted(const RedBuf& rb, int s0) const {
+    return RedBuf{rb.partials + (size_t)s0 * rb.pstride, rb.tickets + s0, rb.pstride,
+                  rb.hist ? rb.hist + (size_t)s0 * kHist * 2 : nullptr};
   }
 
-  // One CG iteration (k1, k2, k3).  A sampled iteration is bracketed by
-  // events, and its stencil kernels count the systems they compute; the
-  // algorithmic bytes of a launch (every stored element touched once) are the
-  // links (and transports) once plus, per computed system, the vectors read
-  // and written: k1 p read, t written; k2 t read, r read and written.
-  void iterate(bool sample, bool count = true) {
+  template <int NS> void launch_k12(const Range& q, cudaStream_t s, int* c) {
+    SysState* S = ws_.S + q.s0;
+    const VF p = shifted(fp_, q.s0 * vunits_), t = shifted(ft_, q.s0 * vunits_);
+    const RedBuf rb = shifted(rb_, q.s0);
+    const dim3 grid1 = gfast_ ? dim3(q.ngrp, q.g1) : dim3(q.g1, q.ngrp),
+               grid2 = gfast_ ? dim3(q.ngrp, q.g2) : dim3(q.g2, q.ngrp);
+    prepass(opf_, p, vunits_, ST_RUNNING, false, s, q.s0, q.n);
+    cg_k1<TF, OpF, NS, GK><<<grid1, kTile, 0, s>>>(gk_, opf_, p, t, bp_, q.n, S, rb, c, gfast_);
+    if (c) cudaEventRecord(samples_.back().e1, s);
+    prepass(opf_, t, vunits_, ST_RUNNING, true, s, q.s0, q.n);
+    cg_k2<TF, OpF, NS, VR, GK><<<grid2, kTile, 0, s>>>(gk_, opf_, t, shifted(fr_, q.s0 * runits_), bp_, q.n, S, rb,
+                                                       c ? c + 1 : nullptr, gfast_);
+  }
+
+  // One CG iteration (k1, k2, k3) of a range.  A sampled iteration (of the
+  // whole batch) is bracketed by events, and its stencil kernels count the
+  // systems they compute; the algorithmic bytes of a launch (every stored
+  // element touched once) are the links (and transports) once plus, per
+  // computed system, the vectors read and written: k1 p read, t written; k2 t
+  // read, r read and written.
+  void iterate(const Range& q, cudaStream_t s, bool sample, bool count = true) {
     SysState* S = ws_.S;
     int* c = nullptr;
     if (sample) {
       samples_.push_back(Sample{prof_event(), prof_event(), prof_event(), prof_event()});
       c = ws_.pcount + 3 * (samples_.size() - 1);
-      cudaEventRecord(samples_.back().e0, ist_);
+      cudaEventRecord(samples_.back().e0, s);
     }
-    commit_ready<<<(cap_ + 127) / 128, 128, 0, ist_>>>(cap_, S);
     if constexpr (MIXED) {
-      if (ns_ == 2) launch_k12<2>(c);
-      else if (ns_ == 4) launch_k12<4>(c);
-      else launch_k12<1>(c);
+      if (ns_ == 2) launch_k12<2>(q, s, c);
+      else if (ns_ == 4) launch_k12<4>(q, s, c);
+      else launch_k12<1>(q, s, c);
     } else {
       if (!use_quad<OpF>(g_.V)) {
-        if constexpr (!quad_always<OpF>()) launch_k12<1>(c);
+        if constexpr (!quad_always<OpF>()) launch_k12<1>(q, s, c);
       } else if constexpr (has_quad<OpF>()) {
-        iter_quad<1, OpF><<<dim3(g1_, cap_), kTile, 0, ist_>>>(g_, opf_, fp_, ft_, vunits_, vunits_, r_, S, rb_, c);
-        if (c) cudaEventRecord(samples_.back().e1, ist_);
-        iter_quad<2, OpF><<<dim3(g2_, cap_), kTile, 0, ist_>>>(g_, opf_, ft_, fr_, vunits_, runits_, r_, S, rb_,
-                                                               c ? c + 1 : nullptr);
+        iter_quad<1, OpF><<<dim3(q.g1, cap_), kTile, 0, s>>>(g_, opf_, fp_, ft_, vunits_, vunits_, r_, S, rb_, c);
+        if (c) cudaEventRecord(samples_.back().e1, s);
+        iter_quad<2, OpF><<<dim3(q.g2, cap_), kTile, 0, s>>>(g_, opf_, ft_, fr_, vunits_, runits_, r_, S, rb_,
+                                                            c ? c + 1 : nullptr);
       }
     }
-    if (sample) cudaEventRecord(samples_.back().e2, ist_);
-    launch_k3(gV_, ST_RUNNING, 3, ist_, c ? c + 2 : nullptr);
-    if (sample) cudaEventRecord(samples_.back().e3, ist_);
+    if (sample) cudaEventRecord(samples_.back().e2, s);
+    launch_k3(q.gV, ST_RUNNING, 3, s, c ? c + 2 : nullptr, q.s0, q.n);
+    if (sample) cudaEventRecord(samples_.back().e3, s);
     if (count) {
-      launches(4);
+      launches(3);
       if (prof()) {
         prof_count(cls_k1(), 1);
         prof_count(cls_k2(), 1);
@@ -1083,11 +1177,14 @@ class Engine {
   SysState* hrd_ = nullptr;   // device alias of hr_ when mapped
   SysState* hstd_ = nullptr;  // device alias of hst_ when mapped
   cudaStream_t st_;
-  cudaStream_t ist_;  // stream the iteration kernels go to (st_, or the loop body's capture stream)
   cudaEvent_t ev_;
   size_t n_;    // complex components of one system's field (g.V x NC)
   size_t s64_;  // per-system stride of the FP64 vectors (n_, or 2 n_ with a two-pass operator's scratch)
-  int ntiles_ = 0, pstride_ = 0, ngrp_ = 0, gV_ = 0, g1_ = 0, g2_ = 0;
+  int ntiles_ = 0, pstride_ = 0, ngrp_ = 0;
+  Range whole_, half_[2];  // the batch, and its halves
+  bool split_ = false;     // the next chunk runs as two halves
+  cudaStream_t half_st_ = nullptr;
+  cudaEvent_t ev_split_ = nullptr, ev_meet_ = nullptr;
   RedBuf rb_{}, rbu_{};
   cudaStream_t side_ = nullptr;  // reliable updates overlapped with iterations
   cudaEvent_t ev_fork_ = nullptr, ev_join_ = nullptr;
@@ -1109,13 +1206,16 @@ class Engine {
     else return (const void*)cg_k3<TF, VR, VF, NC>;
   }
   static int k3_rows(int nsys) { return is_paired<VF>::value ? (nsys + 1) / 2 : nsys; }
-  void launch_k3(int gx, int status, int mode, cudaStream_t s, int* nact) const {
+  void launch_k3(int gx, int status, int mode, cudaStream_t s, int* nact, int s0 = 0, int n = -1) const {
+    if (n < 0) n = cap_;
+    const VR r = shifted(fr_, s0 * runits_), x = shifted(fx_, s0 * runits_);
+    const VF p = shifted(fp_, s0 * vunits_);
     if constexpr (is_paired<VF>::value)
-      cg_k3_pair<VR, VF, NC><<<dim3(gx, k3_rows(cap_)), 256, 0, s>>>(g_.V, fr_, fp_, fx_, runits_, vunits_, ws_.S,
-                                                                     cap_, status, mode, nact);
+      cg_k3_pair<VR, VF, NC><<<dim3(gx, k3_rows(n)), 256, 0, s>>>(g_.V, r, p, x, runits_, vunits_, ws_.S + s0, n,
+                                                                  status, mode, nact);
     else
-      cg_k3<TF, VR, VF, NC><<<dim3(gx, cap_), 256, 0, s>>>(g_.V, fr_, fp_, fx_, runits_, vunits_, ws_.S, status,
-                                                           mode, nact);
+      cg_k3<TF, VR, VF, NC><<<dim3(gx, n), 256, 0, s>>>(g_.V, r, p, x, runits_, vunits_, ws_.S + s0, status, mode,
+                                                        nact);
   }
   // (lanes: threads a site)
   int grid_of(const void* kernel, int block, int nsys, int lanes = 1, int over = 1) const {
@@ -1137,8 +1237,8 @@ class Engine {
   void launches(int k) const {
     if (!capturing_) note_launches(k);
   }
-  int cls_ = 0;  // groups the iteration grids are sized for
-  std::vector<std::pair<int, cudaGraphExec_t>> gexecs_;
+  long long cls_ = 0;  // groups the iteration grids are sized for (two halves: both numbers)
+  std::vector<std::pair<long long, cudaGraphExec_t>> gexecs_;
   std::vector<int> staged_;
   std::vector<char> reported_;
 };
