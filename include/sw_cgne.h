@@ -208,8 +208,10 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  * SW_PARAM_CHUNK: CG iterations launched between two reads of the per-system
  *   status words (1..4096, default 4).  Larger chunks mean fewer host
  *   synchronisations; converged systems idle for at most one chunk, and a
- *   system whose reliable update ran beside a chunk resumes at an iteration
- *   boundary within it.
+ *   system whose reliable update ran beside a chunk resumes with the next one.
+ *   Mixed-precision solves on lattices that a few hundred warps hold (at 152
+ *   SMs: Wilson up to 29184 sites, even-odd twice that, staggered Wilson
+ *   14592) run up to 512 iterations in one launch instead.
  * SW_PARAM_RELIABLE_DELTA: mixed precision only; the FP32 correction is
  *   folded into the FP64 solution and r = b - A x recomputed in FP64 when the
  *   iterated |r| falls below delta times its maximum since the last such
@@ -245,8 +247,10 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  *   synchronisation per call, with results bit-identical to the host-driven
  *   rounds.  Its grids are sized for every system of the batch.  0 (default)
  *   reads the status words on the host after every round.  Solves taken while
- *   kernel timing is enabled (sw_profile_enable), the server's engines and
- *   cgne_solve_noalloc always use the host-driven rounds.
+ *   kernel timing is enabled (sw_profile_enable), the server's engines,
+ *   cgne_solve_noalloc and mixed-precision solves on the small lattices above
+ *   (whose iterations are one launch as it is) always use the host-driven
+ *   rounds.
  * SW_PARAM_WILSON_LEAN: form of the spin-projected (r = 1) FP32 Wilson
  *   stencil: -1 (default) chooses by lattice size -- the lean form (fewer
  *   live registers, 8 blocks per SM) when the packed FP32 links take at most
@@ -310,6 +314,8 @@ int sw_autotune_layout(const sw_lattice* lat, int op, const void* U, const void*
  * profiling is enabled -- timed or not, graph replays included -- is counted
  * as "issued" (sw_profile_issued), so the time a class takes in a solve is
  * its mean time per timed launch times its issued launches.
+ * The one-launch iterations of small lattices (SW_PARAM_CHUNK above) have no
+ * k1, k2 and k3 launches to time; their FP64 classes are recorded as always.
  * Process-wide and thread-safe; disabled by default. */
 int sw_profile_enable(int on);
 /* FP64 fused multiply-add throughput of the current device in TFLOP/s, into

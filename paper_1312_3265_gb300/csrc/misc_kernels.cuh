@@ -260,11 +260,12 @@ static __global__ void mark_ready(int nsys, SysState* S) {
   if (i < nsys && S[i].status == ST_JUST_UPDATED) S[i].status = ST_READY;
 }
 
-// First launch of every CG iteration, on the iteration stream: READY ->
+// First launch of a chunk of CG iterations, on the iteration stream: READY ->
 // RUNNING.  A reliable update running concurrently on another stream marks
 // its systems READY only after all its writes (x, r, p) are complete, and the
-// switch happens between iterations, so every kernel of an iteration sees the
-// same set of running systems.
+// switch happens between chunks, so every kernel of an iteration sees the
+// same set of running systems.  (As the first launch of every iteration it cost
+// a launch each; a system waits at most a chunk, as it does for its update.)
 static __global__ void commit_ready(int nsys, SysState* S) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nsys && S[i].status == ST_READY) S[i].status = ST_RUNNING;
