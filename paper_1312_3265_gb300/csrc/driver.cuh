@@ -73,7 +73,12 @@ constexpr int kOver64 = 8;  // waves of blocks of the FP64 kernels
 // 256 / 237; FP16 12^3x24 38.9 / 33.9; even-odd 16^3x32, 12: 42.2 / 39.8;
 // staggered Wilson 16^4, 12 (57 MB): 17.0 / 15.6 -- but 16^3x32, 24 (113 MB): 52.3
 // / 54.0 and 24^3x48, 24 (573 MB): 252 / 258; Wilson 24^3x48 (191 MB) 358 / 356.
-constexpr double kSplitWork = 1 << 21, kSplitGauge = 80e6;
+// FP64 iterations (bound by the FP64 pipe, so the tails of their launches and k3
+// cost time on any lattice): from 2^14, where a half still fills the chip, whatever
+// the gauge data take.  ms: Wilson 8^3x16, 12 systems 60.2 / 55.3, 2 systems 15.0 /
+// 13.9; 4^3x8, 12: 10.3 / 9.6; 16^3x32, 5: 396 / 368; staggered Wilson 8^4, 3:
+// 3.93 / 3.82; 16^4, 3: 35.9 / 33.9; even-odd 8^3x16, 12: 24.6 / 21.8.
+constexpr double kSplitWork = 1 << 21, kSplitGauge = 80e6, kSplitWork64 = 1 << 14;
 
 // over: waves of blocks at most.  Kernels bound by the FP64 pipe take several:
 // blocks that share the pipe do not run in rounds, and a block that loops over
@@ -369,7 +374,7 @@ class Engine {
     whole_.n = cap;
     whole_.ngrp = ngrp_;
     // halves of whole groups (and pairs)
-    half_[0].n = half_[1].s0 = (ngrp_ + 1) / 2 * ns_ & ~1;
+    half_[0].n = half_[1].s0 = (ngrp_ + 1) / 2 * ns_ & (MIXED ? ~1 : ~0);
     half_[1].n = cap - half_[0].n;
     for (Range& h : half_) h.ngrp = (h.n + ns_ - 1) / ns_;
     cls_ = ngrp_;
@@ -418,7 +423,7 @@ class Engine {
         cudaGetLastError();
         side_ = nullptr;
       }
-      if (MIXED && !small_ && cap_ >= 2 * std::max(2, ns_) &&
+      if (!small_ && cap_ >= (MIXED ? 2 * std::max(2, ns_) : 2) &&
           (cudaStreamCreateWithFlags(&half_st_, cudaStreamNonBlocking) != cudaSuccess ||
            cudaEventCreateWithFlags(&ev_split_, cudaEventDisableTiming) != cudaSuccess ||
            cudaEventCreateWithFlags(&ev_meet_, cudaEventDisableTiming) != cudaSuccess)) {
@@ -982,9 +987,10 @@ class Engine {
   // A chunk of iterations on the engine's stream -- or as two halves of the
   // slots on two streams, which share nothing but the gauge field: one half's
   // streaming k3 (bound by memory) and the tails of its launches then run
-  // beside the other's stencils (bound by the loads in flight).
+  // beside the other's stencils (bound by the loads in flight).  A chunk whose
+  // kernels are timed runs whole: its events time each kernel alone.
   void run_chunk(bool sample, bool count) {
-    if (split_) {
+    if (split_ && !sample) {
       cudaEventRecord(ev_split_, st_);
       cudaStreamWaitEvent(half_st_, ev_split_, 0);
       commit(half_[0], st_);
@@ -1045,18 +1051,18 @@ class Engine {
   // them that a half's launches are longer than the host takes to issue two.
   void size_for_live() {
     int n0 = 0, n1 = 0;
-    const bool may = half_st_ && !prof() && (double)g_.V * OpF::kGaugeBytes <= kSplitGauge;
+    const bool may = half_st_ && (!MIXED || (double)g_.V * OpF::kGaugeBytes <= kSplitGauge);
     const int a = may ? live_class(half_[0], &n0) : 0, b = a ? live_class(half_[1], &n1) : 0;
-    split_ = a && b && (double)g_.V * NC * (n0 + n1) >= kSplitWork;
+    split_ = a && b && (double)g_.V * NC * (n0 + n1) >= (MIXED ? kSplitWork : kSplitWork64);
     int n = 0;
-    const long long cls = split_ ? ((long long)a << 32) + b : std::max(1, live_class(whole_, &n));
+    const int w = std::max(1, live_class(whole_, &n));
+    const long long cls = split_ ? ((long long)a << 32) + b : w;
     if (cls == cls_) return;
     cls_ = cls;
+    set_grids(whole_, w);  // (also of the chunks whose kernels are timed)
     if (split_) {
       set_grids(half_[0], a);
       set_grids(half_[1], b);
-    } else {
-      set_grids(whole_, (int)cls);
     }
   }
 
@@ -1125,7 +1131,7 @@ class Engine {
   // computed system, the vectors read and written: k1 p read, t written; k2 t
   // read, r read and written.
   void iterate(const Range& q, cudaStream_t s, bool sample, bool count = true) {
-    SysState* S = ws_.S;
+    SysState* S = ws_.S + q.s0;
     int* c = nullptr;
     if (sample) {
       samples_.push_back(Sample{prof_event(), prof_event(), prof_event(), prof_event()});
@@ -1140,10 +1146,12 @@ class Engine {
       if (!use_quad<OpF>(g_.V)) {
         if constexpr (!quad_always<OpF>()) launch_k12<1>(q, s, c);
       } else if constexpr (has_quad<OpF>()) {
-        iter_quad<1, OpF><<<dim3(q.g1, cap_), kTile, 0, s>>>(g_, opf_, fp_, ft_, vunits_, vunits_, r_, S, rb_, c);
+        const VF p = shifted(fp_, q.s0 * vunits_), t = shifted(ft_, q.s0 * vunits_);
+        const RedBuf rb = shifted(rb_, q.s0);
+        iter_quad<1, OpF><<<dim3(q.g1, q.n), kTile, 0, s>>>(g_, opf_, p, t, vunits_, vunits_, r_, S, rb, c);
         if (c) cudaEventRecord(samples_.back().e1, s);
-        iter_quad<2, OpF><<<dim3(q.g2, cap_), kTile, 0, s>>>(g_, opf_, ft_, fr_, vunits_, runits_, r_, S, rb_,
-                                                            c ? c + 1 : nullptr);
+        iter_quad<2, OpF><<<dim3(q.g2, q.n), kTile, 0, s>>>(g_, opf_, t, shifted(fr_, q.s0 * runits_), vunits_, runits_,
+                                                           r_, S, rb, c ? c + 1 : nullptr);
       }
     }
     if (sample) cudaEventRecord(samples_.back().e2, s);
@@ -1151,7 +1159,7 @@ class Engine {
     if (sample) cudaEventRecord(samples_.back().e3, s);
     if (count) {
       launches(3);
-      if (prof()) {
+      if (prof() && q.s0 == 0) {  // (two halves of an iteration: as one)
         prof_count(cls_k1(), 1);
         prof_count(cls_k2(), 1);
         prof_count(cls_k3(), 1);

@@ -2,7 +2,7 @@
 system against its solve alone (never split), bit for bit.
 
 The batches are just above and below the work from which chunks split (2^21
-complex numbers in a vector of the running systems), with odd numbers of systems
+complex numbers in a vector of the running systems, FP64 mode 2^14), with odd numbers of systems
 and masses far apart, so that the halves empty at different times and the chunk
 falls back to a whole one on the way.
 """
@@ -27,7 +27,9 @@ def sw():
 
 @pytest.mark.parametrize("op,prec,dims,nsys", [
     ("wilson", 1, (12, 12, 12, 24), 4), ("wilson", 1, (12, 12, 12, 24), 5), ("wilson", 2, (12, 12, 12, 24), 7),
-    ("wilson_eo", 1, (14, 14, 14, 26), 5), ("sw", 1, (16, 16, 16, 16), 11), ("sw", 2, (14, 16, 16, 18), 13)])
+    ("wilson_eo", 1, (14, 14, 14, 26), 5), ("sw", 1, (16, 16, 16, 16), 11), ("sw", 2, (14, 16, 16, 18), 13),
+    ("wilson", 0, (4, 4, 6, 8), 2), ("wilson", 0, (6, 6, 6, 6), 2), ("wilson", 0, (48, 48, 10, 6), 3),
+    ("wilson_eo", 0, (6, 6, 6, 6), 5), ("sw", 0, (4, 6, 8, 10), 3), ("sw", 0, (6, 6, 10, 10), 7)])
 def test_halves_equal_single_solves(sw, op, prec, dims, nsys):
     import torch
     g = torch.Generator("cuda").manual_seed(11)
