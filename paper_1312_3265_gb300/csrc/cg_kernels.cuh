@@ -56,6 +56,7 @@ struct SysState {
   double cb2;      // |b|^2 of the convergence criterion when it is another system's (0: b2)
   double rmax2;    // max |r|^2 since the last reliable update
   double delta2;   // reliable-update trigger factor (0: only at convergence)
+  double delta;    // reduction of the residual a leg is to take (0: FP64 mode)
   double rr_true;  // last FP64 residual norm^2
   double x02;      // |x0|^2 of the initial guess
   double mass;     // bare mass of this system
@@ -454,6 +455,20 @@ __device__ __forceinline__ void finish_k2(SysState& st, const RedBuf& rb, int sy
     if (rr <= st.trig2 || st.iter >= st.max_iter || rr < st.delta2 * st.rmax2) st.status = ST_NEED_RU;
   }
 }
+// Reliable-update trigger of the legs that remain after an update that did not
+// converge: the fewest that reduce the residual from rr to the check's trigger
+// by about `delta` each, made equal (driver.cuh, leg_delta).  Planned from the
+// residual the update found: the first legs are cut at the tolerance and at the
+// largest |r|, and a residual that grew before it fell, or the even-odd
+// operator's lower trigger, would end the last leg just above the trigger and
+// cost one more FP64 residual.
+static __device__ __noinline__ void plan_legs(SysState& s, double rr) {
+  if (s.delta <= 0.0) return;
+  const double target = 0.5 * log(fmax(s.trig2, 1e-300) / rr);
+  const double legs = ceil(target / log(s.delta) - 0.25);
+  s.delta2 = legs > 1.0 ? exp(2.0 * target / legs) : 0.0;
+}
+
 // the FP64 residual's: converged, out of iterations, or on with the new residual
 __device__ __forceinline__ void finish_residual(SysState& s, const RedBuf& rb, int sys, double rr) {
   s.rr_true = rr;
@@ -469,6 +484,7 @@ __device__ __forceinline__ void finish_residual(SysState& s, const RedBuf& rb, i
     record(rb, sys, s.iter - 1, 1, s.beta);
     s.rr = rr;
     s.rmax2 = rr;
+    plan_legs(s, rr);
     s.status = ST_JUST_UPDATED;
   }
 }
@@ -761,6 +777,7 @@ __global__ void __launch_bounds__(kTile) residual64(Geom g, Op op, typename Op::
         record(rb, sys, s.iter - 1, 1, s.beta);
         s.rr = rr;
         s.rmax2 = rr;
+        plan_legs(s, rr);
         s.status = ST_JUST_UPDATED;
       }
     }

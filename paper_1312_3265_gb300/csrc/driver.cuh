@@ -195,7 +195,8 @@ inline double* pinned_hist(size_t n) {
 // short last leg, whose FP64 residual costs as much as the others'.  A leg may
 // go a quarter (in the logarithm) below delta where that saves one: at 3e-5
 // FP32 iterations keep their count down to 1e-5.  tol 1e-8: 2 legs of 1e-4;
-// 1e-10: 2 of 1e-5 (by 3e-5: 3); 1e-12: 3 of 1e-4.
+// 1e-10: 2 of 1e-5 (by 3e-5: 3); 1e-12: 3 of 1e-4.  An update that does not
+// converge plans the legs that remain (cg_kernels.cuh, plan_legs).
 inline double leg_delta(double tol, double delta) {
   const double legs = std::max(1.0, std::ceil(std::log(tol) / std::log(delta) - 0.25));
   return std::pow(tol, 1.0 / legs);
@@ -542,6 +543,7 @@ class Engine {
     s.cb2 = cb2;
     const double leg = MIXED ? leg_delta(tol, delta_) : 0.0;
     s.delta2 = leg * leg;
+    s.delta = MIXED ? delta_ : 0.0;
     s.max_iter = max_iter;
     s.mass = mass;
     s.status = ST_ADMIT;
