@@ -184,11 +184,13 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, nt = gridDim.x;
   const unsigned long long tag = (unsigned long long)epoch << 32;
   unsigned long long* slots = a.slots + (size_t)(PHASE - 1) * a.nsys * nt * nt * 2;
+  // The block's stores, before any of its words: by every warp that may post
+  // one, whichever of its systems still run.
+  if ((int)(threadIdx.x >> 5) < share) fence_gpu();
   for (int t = threadIdx.x >> 5; t < share; t += nw) {
     if (!s.on[t]) continue;
     double v = s.wsum[t][0];
     for (int w = 1; w < nw; ++w) v += s.wsum[t][w];
-    if (t < nw) fence_gpu();  // the block's stores, before its words
     const unsigned long long hi = tag | (unsigned)__double2hiint(v), lo = tag | (unsigned)__double2loint(v);
     for (int i = lane; i < nt; i += 32) st_relaxed(slots + (((size_t)s.sys[t] * nt + i) * nt + blockIdx.x) * 2, hi, lo);
   }

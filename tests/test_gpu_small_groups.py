@@ -1,0 +1,69 @@
+"""The one-launch iterations of small lattices (small.cuh) with many systems in a
+group of blocks: more than two a warp of a block, those that stop first (heavy
+masses) at the front of the batch, so that every warp's first systems have
+stopped while most of the group runs on; and more systems than the groups
+resident at once hold, so that a round takes several launches.  Every system is
+compared bit for bit with its solve alone, and the batch with itself.
+"""
+import pytest
+
+import lattice_synth as ls
+
+pytestmark = pytest.mark.gpu
+
+OPS = {"sw": 0, "wilson": 1, "wilson_eo": 2}
+
+
+@pytest.fixture(scope="module")
+def sw():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1312_3265_gb300 as m
+    m.lib()
+    return m
+
+
+def su3_field(V, g):
+    """SU(3): unitary factor of a Gaussian near 1, its determinant's phase divided out."""
+    import torch
+    z = torch.eye(3, dtype=torch.complex128, device="cuda") + 0.3 * torch.randn(
+        (V * 4, 3, 3), dtype=torch.complex128, device="cuda", generator=g)
+    Q, R = torch.linalg.qr(z)
+    d = torch.diagonal(R, dim1=-2, dim2=-1)
+    Q = Q * (d / d.abs())[:, None, :]
+    return (Q / torch.linalg.det(Q)[:, None, None] ** (1.0 / 3.0)).reshape(V, 4, 3, 3).contiguous()
+
+
+# with 152 SMs: 6 warps a block and 2 groups; 12 warps, one group, two launches
+# (70 systems); 9 warps, one group; staggered Wilson 6 warps, 3 groups; 12 warps,
+# one group, two launches
+@pytest.mark.parametrize("op,prec,dims,nsys", [
+    ("wilson", 1, (6, 10, 12, 14), 48), ("wilson", 2, (6, 10, 12, 14), 48), ("wilson", 1, (12, 12, 12, 16), 70),
+    ("wilson_eo", 1, (12, 12, 12, 24), 40), ("sw", 1, (8, 8, 8, 8), 61), ("sw", 2, (8, 8, 8, 8), 61),
+    ("sw", 1, (8, 8, 8, 28), 75)])
+def test_many_systems_a_group(sw, op, prec, dims, nsys):
+    import torch
+    g = torch.Generator("cuda").manual_seed(17)
+    V = ls.volume(dims)
+    U = su3_field(V, g)
+    W = None
+    if op == "sw":
+        W = torch.empty((V, 8, 3, 3), dtype=torch.complex128, device="cuda")
+        sw.sw_hypercube_build(dims, U, W, False)
+    chi = torch.randn((nsys, V) + ((3,) if op == "sw" else (4, 3)), dtype=torch.complex128, device="cuda", generator=g)
+    heavy = (nsys + 2) // 3
+    masses = [4.0] * heavy + [0.1 + 0.2 * k / nsys for k in range(nsys - heavy)]
+    ref = None
+    for _ in range(3):
+        x = torch.zeros_like(chi)
+        rc, infos = sw.cgne_solve_batch(dims, OPS[op], U, W, chi, x, masses, 1.0, 1e-9, 5000, prec, False)
+        assert rc == sw.SW_OK and all(i.true_rel_resid <= 1e-9 for i in infos)
+        ref = x if ref is None else ref
+        assert torch.equal(x, ref)
+    assert max(i.iters for i in infos[:heavy]) < min(i.iters for i in infos[heavy:])
+    for k, m in enumerate(masses):
+        one = torch.zeros_like(chi[k])
+        info = sw.cgne_solve(dims, OPS[op], U, W, chi[k].contiguous(), one, m, 1.0, 1e-9, 5000, prec, False)
+        assert info.iters == infos[k].iters and info.reliable_updates == infos[k].reliable_updates
+        assert torch.equal(one, x[k])
