@@ -394,8 +394,7 @@ class Engine {
           cudaGetLastError();
           small_ = false;
         } else {
-          cudaMemsetAsync(ws.slots, 0, 8 * small_slots(g.V, cap), st);
-          cudaMemsetAsync(ws.list, 0, sizeof(int) * small_words(g.V, cap), st);
+          clear_small();
         }
       }
     }
@@ -908,6 +907,12 @@ class Engine {
     launches(MIXED ? 7 : 5);
   }
 
+  // The small-lattice kernels' list, "gave up" words and inboxes, zeroed.
+  void clear_small() {
+    cudaMemsetAsync(ws_.slots, 0, 8 * small_slots(g_.V, cap_), st_);
+    cudaMemsetAsync(ws_.list, 0, sizeof(int) * small_words(g_.V, cap_), st_);
+  }
+
   // Small lattices: many iterations of every running system by one launch (a
   // launch a window of the list, where the batch exceeds the blocks resident).
   void iterate_small() {
@@ -920,13 +925,13 @@ class Engine {
       splan_.groups = std::max(1, std::min(units, small_blocks_[splan_.wide] / splan_.tiles));
       splan_.windows = (bound * per + splan_.groups * kSmallShare - 1) / (splan_.groups * kSmallShare);
       unsigned* bad = reinterpret_cast<unsigned*>(ws_.list + cap_ + 1);
+      if (small_epochs_.restart()) clear_small();
       build_list<<<1, 256, 0, st_>>>(cap_, ws_.S, ws_.list, bad, splan_.groups, per);
       for (int w = 0; w < splan_.windows; ++w) {
         launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
-                     SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epoch_, w,
-                               splan_.windows},
+                     SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epochs_.take(),
+                               w, splan_.windows},
                      splan_, st_);
-        small_epoch_ += 8 * kSmallIters;
       }
       launches(1 + splan_.windows);
     }
@@ -1236,7 +1241,7 @@ class Engine {
   bool small_ = false;  // the whole iteration in one cooperative kernel (small.cuh)
   SmallPlan splan_;
   int small_blocks_[2] = {0, 0};  // blocks of its two forms resident at once
-  unsigned small_epoch_ = 0;  // barrier epochs used so far
+  BarrierEpochs small_epochs_;
   std::vector<Sample> samples_;
   std::vector<FpSample> fsamples_;
   long long rounds_ = 0, chunks_ = 0;

@@ -41,6 +41,7 @@
 #include <algorithm>
 
 #include "cg_kernels.cuh"
+#include "epochs.h"
 #include "internal.h"
 
 namespace swc {
@@ -55,6 +56,7 @@ constexpr int kSmallWide = 256;     // largest block of the 255-register form
 constexpr int kSmallWarps = 6;
 constexpr int kSmallShare = 64;     // systems a group of blocks holds
 constexpr int kSmallIters = 512;    // iterations a launch at most
+static_assert(5 * kSmallIters < BarrierEpochs::kLaunch, "epochs of a launch (even-odd: 5 an iteration)");
 constexpr int kWaitLimit = 1 << 22;
 
 // Units (systems, or pairs of them) that run, in order: list[0] = their

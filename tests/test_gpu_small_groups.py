@@ -67,3 +67,35 @@ def test_many_systems_a_group(sw, op, prec, dims, nsys):
         info = sw.cgne_solve(dims, OPS[op], U, W, chi[k].contiguous(), one, m, 1.0, 1e-9, 5000, prec, False)
         assert info.iters == infos[k].iters and info.reliable_updates == infos[k].reliable_updates
         assert torch.equal(one, x[k])
+
+
+def test_long_lived_engine(sw):
+    """A server engine that has run more launches of the small-lattice kernel
+    than its inboxes keep epochs for (1024), with one group of blocks, then
+    takes a burst of many groups: every result equals the solve's, bit for bit."""
+    import torch
+    dims, slots = (4, 4, 4, 4), 96
+    V = ls.volume(dims)
+    g = torch.Generator("cuda").manual_seed(5)
+    U = su3_field(V, g)
+    chi = torch.randn((slots, V, 4, 3), dtype=torch.complex128, device="cuda", generator=g).cpu().pin_memory()
+    x = torch.zeros_like(chi).pin_memory()
+    srv = sw.Server(4 << 30)
+    try:
+        e = srv.add_engine(dims, sw.SW_OP_WILSON, U, slots=slots)
+        for i in range(1100):  # each takes a launch at least
+            srv.submit(e, chi[0], x[0], 4.0, 1e-2)
+            srv.drain()
+            (_, info), = srv.poll()
+            assert info.status == sw.SW_OK
+        masses = [0.1 + 0.01 * k for k in range(slots)]
+        ids = {srv.submit(e, chi[k], x[k], m, 1e-9): k for k, m in enumerate(masses)}
+        srv.drain()
+        for rid, info in srv.poll():
+            k = ids[rid]
+            one = torch.zeros((V, 4, 3), dtype=torch.complex128, device="cuda")
+            ref = sw.cgne_solve(dims, sw.SW_OP_WILSON, U, None, chi[k].cuda(), one, masses[k], 1.0, 1e-9, 100000,
+                                sw.SW_PREC_F32_RELIABLE)
+            assert info.iters == ref.iters and torch.equal(one.cpu(), x[k])
+    finally:
+        srv.close()
