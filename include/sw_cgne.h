@@ -258,12 +258,18 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  *   always the default form.  The two forms perform the same operations in
  *   the same order: results are bit-identical, only the speed differs.  Read
  *   when a solve starts or a server engine is created.
+ * SW_PARAM_WAIT_POLLS: polls (of about a microsecond) after which a wait
+ *   between the blocks of a one-launch iteration (the small lattices above)
+ *   gives up (1..2^30, default 2^22).  The launch then ends, and the systems it
+ *   held end with SW_ERR_TIMEOUT; their x is that of the last FP64 residual.
+ *   Read when a solve starts or a server engine is created.
  * None of these changes what a solve converges to: convergence is always
  * decided on an FP64 residual.  Returns SW_ERR_ARG for an unknown key or a
  * value out of range. */
 enum { SW_PARAM_CHUNK = 0, SW_PARAM_RELIABLE_DELTA = 1, SW_PARAM_NS_SW = 2, SW_PARAM_NS_WILSON = 3,
        SW_PARAM_GRAPHS = 4, SW_PARAM_SITE_BLOCKING = 5, SW_PARAM_GROUP_FAST = 6,
-       SW_PARAM_RELIABLE_DELTA_F16 = 9, SW_PARAM_PERSISTENT = 10, SW_PARAM_WILSON_LEAN = 11 };
+       SW_PARAM_RELIABLE_DELTA_F16 = 9, SW_PARAM_PERSISTENT = 10, SW_PARAM_WILSON_LEAN = 11,
+       SW_PARAM_WAIT_POLLS = 12 };
 enum { SW_SITE_SHAPES = 6 };
 int sw_set_param(int key, double value);
 int sw_get_param(int key, double* value);

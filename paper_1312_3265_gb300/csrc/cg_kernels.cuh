@@ -40,7 +40,8 @@ enum SysStatus : int {
   ST_ZERO_B = 8,        // admitted with b = 0: solution x = 0
   ST_ZERO_GUESS = 9,    // admitted with x0 = 0: r = b, no matvec needed
   ST_RU_PENDING = 10,   // taken into this round's reliable update (from NEED_RU)
-  ST_READY = 11         // residual replaced and p refreshed: runs from the next iteration
+  ST_READY = 11,        // residual replaced and p refreshed: runs from the next iteration
+  ST_GAVE_UP = 12       // a wait between blocks gave up (small.cuh): ended without a result
 };
 
 // Plain data of 8-byte words (moved between device and host as such).

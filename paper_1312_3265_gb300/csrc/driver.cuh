@@ -42,6 +42,7 @@ int param_ns(int nc);  // systems per thread of the FP32 stencils (1, 2 or 4) fo
 bool param_group_fast();     // system groups as the fastest grid dimension of the stencils
 bool param_graphs();   // replay chunks of iterations as captured CUDA graphs
 bool param_persistent();  // whole solve as one CUDA graph with a device-driven loop of rounds
+int param_wait_polls();  // polls after which a wait of the small-lattice kernels gives up
 int param_wilson_lean();  // -1 by lattice size, 0 the default form, 1 the lean form (FP32 Wilson, r = 1)
 
 // Operators applied in two passes (the even-odd Schur complement): before
@@ -436,6 +437,7 @@ class Engine {
     hstd_ = mapped_alias(hst_);
     move_states(ws.S, hr_, hrd_, cap, cudaMemcpyHostToDevice);
     chunk_ = param_chunk();
+    polls_ = param_wait_polls();
     delta_ = param_delta(std::is_same<VF, VecP16<NC>>::value);
   }
 
@@ -646,7 +648,7 @@ class Engine {
   void finished(std::vector<int>& out) {
     for (int i = 0; i < cap_; ++i) {
       const int s = hr_[i].status;
-      if (!reported_[i] && (s == ST_CONVERGED || s == ST_MAXITER || s == ST_FAILED)) {
+      if (!reported_[i] && (s == ST_CONVERGED || s == ST_MAXITER || s == ST_FAILED || s == ST_GAVE_UP)) {
         reported_[i] = 1;
         out.push_back(i);
       }
@@ -930,7 +932,7 @@ class Engine {
       for (int w = 0; w < splan_.windows; ++w) {
         launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
                      SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epochs_.take(),
-                               w, splan_.windows},
+                               w, splan_.windows, polls_},
                      splan_, st_);
       }
       launches(1 + splan_.windows);
@@ -1242,6 +1244,7 @@ class Engine {
   SmallPlan splan_;
   int small_blocks_[2] = {0, 0};  // blocks of its two forms resident at once
   BarrierEpochs small_epochs_;
+  int polls_ = 1;
   std::vector<Sample> samples_;
   std::vector<FpSample> fsamples_;
   long long rounds_ = 0, chunks_ = 0;

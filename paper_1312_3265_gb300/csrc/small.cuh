@@ -26,8 +26,8 @@
 // system 255, all hops' loads under way at once); the blocks of a group of
 // systems wait on one another only, and the launch is cooperative, so they are
 // resident together.
-// A wait gives up after kWaitLimit polls: the group's systems are then handed
-// to a reliable update (any x is a valid guess) and the launch ends.
+// A wait gives up after SW_PARAM_WAIT_POLLS polls: the launch ends, and the
+// group's systems end without a result (ST_GAVE_UP, SW_ERR_TIMEOUT to the caller).
 //
 // An iteration of one system takes 12-14 us, of which the hops are 4, the FP64
 // sums and divisions 3-4 and the fences and inboxes 5.  Measured against the
@@ -57,7 +57,6 @@ constexpr int kSmallWarps = 6;
 constexpr int kSmallShare = 64;     // systems a group of blocks holds
 constexpr int kSmallIters = 512;    // iterations a launch at most
 static_assert(5 * kSmallIters < BarrierEpochs::kLaunch, "epochs of a launch (even-odd: 5 an iteration)");
-constexpr int kWaitLimit = 1 << 22;
 
 // Units (systems, or pairs of them) that run, in order: list[0] = their
 // number, list[1 + i] = (unit << 2) | mask of the unit's systems; systems in
@@ -105,6 +104,7 @@ struct SmallArgs {
   unsigned* bad;              // [groups] "gave up"
   unsigned epoch;             // above every epoch of the launches before
   int window, windows;        // this launch's part of the list
+  int polls;                  // polls after which a wait gives up
 };
 
 // ---------------------------------------------------------------- the group's state and barriers
@@ -131,7 +131,7 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
 }
 // one more poll in vain: whether to give up
 __device__ __forceinline__ bool give_up(const SmallArgs& a, SmallShared& s, int& n) {
-  if (++n <= kWaitLimit && ((n & 255) || !ld_relaxed(a.bad + blockIdx.y))) return false;
+  if (++n <= a.polls && ((n & 255) || !ld_relaxed(a.bad + blockIdx.y))) return false;
   atomicExch(a.bad + blockIdx.y, 1u);
   s.ok = 0;
   return true;
@@ -225,6 +225,7 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
   }
   fence_gpu();
   __syncthreads();
+  if (!s.ok) return false;  // (the sums are incomplete)
   // one thread a system: the divisions of all systems at once
   RedBuf rb = a.rb;
   if (blockIdx.x) rb.hist = nullptr;
@@ -241,7 +242,7 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
     if (st.status != ST_RUNNING) s.on[t] = 0;
   }
   __syncthreads();
-  return s.ok != 0;
+  return true;
 }
 
 // The group's part of the list -> shared memory; returns its size (systems).
@@ -277,22 +278,24 @@ __device__ __forceinline__ bool group_goes_on(const SmallShared& s, int share) {
   return on > 0 && 2 * on > all;
 }
 
+// The group's states at the launch's end, by its block 0: what the iterations
+// change, and the status where it is still the one the launch found.  A block
+// whose wait gave up ends its group's systems, whatever the other blocks make of
+// them: block 0 may have passed its last wait before another gave up in its own.
 __device__ __forceinline__ void store_states(const SmallArgs& a, const SmallShared& s, int share, bool gave_up) {
   __syncthreads();
-  if (!gave_up) {
-    if (blockIdx.x) return;
-    gave_up = ld_relaxed(a.bad + blockIdx.y) != 0;  // another block did, at the last barrier
-  }
+  if (!gave_up && blockIdx.x) return;
   for (int t = threadIdx.x; t < share; t += blockDim.x) {
     if (s.sys[t] < 0) continue;
-    if (gave_up) {  // (every block writes the same)
-      SysState& st = a.S[s.sys[t]];
-      st.alpha = 0.0;
-      st.rr_old = __longlong_as_double(0x7ff0000000000000ll);  // beta = 0: the direction starts anew
-      st.status = ST_NEED_RU;
-    } else {
-      a.S[s.sys[t]] = s.st[t];
+    SysState& g = a.S[s.sys[t]];
+    if (gave_up) {
+      atomicExch(&g.status, ST_GAVE_UP);
+      continue;
     }
+    const SysState& l = s.st[t];
+    g.rr = l.rr, g.rr_old = l.rr_old, g.pAp = l.pAp, g.alpha = l.alpha, g.beta = l.beta, g.rmax2 = l.rmax2;
+    g.iter = l.iter;
+    atomicCAS(&g.status, ST_RUNNING, l.status);
   }
 }
 

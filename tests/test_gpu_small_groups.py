@@ -99,3 +99,44 @@ def test_long_lived_engine(sw):
             assert info.iters == ref.iters and torch.equal(one.cpu(), x[k])
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("op,prec", [("sw", 1), ("sw", 2), ("wilson", 1), ("wilson_eo", 1)])
+def test_a_wait_that_gives_up_is_a_timeout(sw, op, prec):
+    """With one poll allowed, a wait for 100 other blocks runs out: the call
+    returns SW_ERR_TIMEOUT at once, for every system of the batch and to a
+    request of a server, and the next calls, with the default limit, solve."""
+    import torch
+    dims, nsys = (8, 8, 8, 16) if op != "wilson_eo" else (8, 8, 16, 16), 3
+    V = ls.volume(dims)
+    g = torch.Generator("cuda").manual_seed(3)
+    U = su3_field(V, g)
+    W = None
+    if op == "sw":
+        W = torch.empty((V, 8, 3, 3), dtype=torch.complex128, device="cuda")
+        sw.sw_hypercube_build(dims, U, W, False)
+    chi = torch.randn((nsys, V) + ((3,) if op == "sw" else (4, 3)), dtype=torch.complex128, device="cuda", generator=g)
+    solve = lambda x: sw.cgne_solve_batch(dims, OPS[op], U, W, chi, x, [0.2, 0.3, 0.4], 1.0, 1e-9, 5000, prec, False)
+    old = sw.sw_get_param(sw.SW_PARAM_WAIT_POLLS)
+    srv = sw.Server(4 << 30)
+    try:
+        sw.sw_set_param(sw.SW_PARAM_WAIT_POLLS, 1)
+        x = torch.zeros_like(chi)
+        before = sw.sw_kernel_launches()
+        with pytest.raises(sw.SWError) as e:
+            solve(x)
+        assert e.value.code == -7
+        assert sw.sw_kernel_launches() - before < 40  # admission and one round
+        if op != "wilson_eo":
+            eng = srv.add_engine(dims, OPS[op], U, precision=prec, slots=2)
+            ch, xh = chi[0].cpu().pin_memory(), torch.zeros_like(chi[0]).cpu().pin_memory()
+            srv.submit(eng, ch, xh, 0.2, 1e-9)
+            srv.drain(60)
+            (_, info), = srv.poll()
+            assert info.status == -7
+    finally:
+        sw.sw_set_param(sw.SW_PARAM_WAIT_POLLS, old)
+        srv.close()
+    x = torch.zeros_like(chi)
+    rc, infos = solve(x)
+    assert rc == sw.SW_OK and all(i.true_rel_resid <= 1e-9 for i in infos)
