@@ -590,9 +590,10 @@ class Engine {
         reliable_update(n_ru, st_, kOver64);
       }
     }
-    if (run && small_) {
-      iterate_small();
-    } else if (run) {
+    // (a cooperative launch that is refused: the rest of the solve, this round's
+    // iterations included, by the kernels of larger lattices)
+    if (run && small_) small_ = iterate_small();
+    if (run && !small_) {
       size_for_live();
       // every 4th chunk is timed when profiling, on its second iteration: by
       // then the queue is full, so the events time the kernels rather than the
@@ -917,7 +918,8 @@ class Engine {
 
   // Small lattices: many iterations of every running system by one launch (a
   // launch a window of the list, where the batch exceeds the blocks resident).
-  void iterate_small() {
+  // False: a launch was refused (the systems of the windows before it have run).
+  bool iterate_small() {
     if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
       constexpr int per = small_traits<OpF>::kPer;
       const int units = std::max(1, (live_slots() + per - 1) / per), bound = (cap_ + per - 1) / per;
@@ -930,13 +932,19 @@ class Engine {
       if (small_epochs_.restart()) clear_small();
       build_list<<<1, 256, 0, st_>>>(cap_, ws_.S, ws_.list, bad, splan_.groups, per);
       for (int w = 0; w < splan_.windows; ++w) {
-        launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
-                     SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epochs_.take(),
-                               w, splan_.windows, polls_},
-                     splan_, st_);
+        const cudaError_t e =
+            launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
+                         SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epochs_.take(),
+                                   w, splan_.windows, polls_},
+                         splan_, st_);
+        launches(w ? 1 : 2);
+        if (e != cudaSuccess) {
+          cudaGetLastError();
+          return false;
+        }
       }
-      launches(1 + splan_.windows);
     }
+    return true;
   }
 
   // Slots that may run in the next chunk.

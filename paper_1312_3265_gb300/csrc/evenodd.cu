@@ -228,10 +228,10 @@ const void* small_kernel(const WEOOp<float, G, VA, R1>&, bool wide) {
   return wilson_small_kernel<R1, HalfSites, G, VA<12>>(wide);
 }
 template <typename G, template <int> class VA, bool R1>
-void launch_small(const WEOOp<float, G, VA, R1>& op, const GeomBlk&, VA<12> p, VA<12> t, VecP32q<12> r, VecP32q<12> x,
-                  const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
-  launch_cooperative(small_kernel(op, pl.wide), pl, st, HalfSites{op.full}, op.U, p, t, r, x,
-                     op.half_units, a);
+cudaError_t launch_small(const WEOOp<float, G, VA, R1>& op, const GeomBlk&, VA<12> p, VA<12> t, VecP32q<12> r,
+                         VecP32q<12> x, const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
+  return launch_cooperative(small_kernel(op, pl.wide), pl, st, HalfSites{op.full}, op.U, p, t, r, x,
+                            op.half_units, a);
 }
 
 // chi^_e = chi_e - D_eo chi_o / M and the even part of the guess, per system,

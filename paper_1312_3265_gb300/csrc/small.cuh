@@ -931,10 +931,12 @@ inline bool small_tiles(int V, int sites_per_warp, SmallPlan* p) {
   return true;
 }
 
+// Refused (an error returned, nothing launched) where the grid cannot be
+// resident, for instance beside a limit on the SMs the process may use.
 template <class... Args>
-void launch_cooperative(const void* kernel, const SmallPlan& p, cudaStream_t st, Args... args) {
+cudaError_t launch_cooperative(const void* kernel, const SmallPlan& p, cudaStream_t st, Args... args) {
   void* v[] = {(void*)&args...};
-  cudaLaunchCooperativeKernel(kernel, dim3(p.tiles, p.groups), dim3(p.nt), v, 0, st);
+  return cudaLaunchCooperativeKernel(kernel, dim3(p.tiles, p.groups), dim3(p.nt), v, 0, st);
 }
 
 // the kernel of an operator (wide: the 255-register form), and its launch
@@ -944,9 +946,9 @@ const void* small_kernel(const SWOp<float, G, Wt, VA>&, bool wide) {
               : (const void*)sw_small<kSmallThreads, GeomBlk, G, Wt, VA<3>>;
 }
 template <typename G, typename Wt, template <int> class VA>
-void launch_small(const SWOp<float, G, Wt, VA>& op, const GeomBlk& g, VA<3> p, VA<3> t, VecP32<3> r, VecP32<3> x,
-                  const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
-  launch_cooperative(small_kernel(op, pl.wide), pl, st, g, op.U, op.W, p, t, r, x, a);
+cudaError_t launch_small(const SWOp<float, G, Wt, VA>& op, const GeomBlk& g, VA<3> p, VA<3> t, VecP32<3> r, VecP32<3> x,
+                         const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
+  return launch_cooperative(small_kernel(op, pl.wide), pl, st, g, op.U, op.W, p, t, r, x, a);
 }
 template <bool R1, class Sites, class GA, class VI> const void* wilson_small_kernel(bool wide) {
   return wide ? (const void*)wilson_small<kSmallWide, R1, Sites, GA, VI>
@@ -957,9 +959,9 @@ const void* small_kernel(const WOp<float, G, VA, R1, LEAN>&, bool wide) {
   return wilson_small_kernel<R1, FullSites<GeomBlk>, G, VA<12>>(wide);
 }
 template <typename G, template <int> class VA, bool R1, bool LEAN>
-void launch_small(const WOp<float, G, VA, R1, LEAN>& op, const GeomBlk& g, VA<12> p, VA<12> t, VecP32q<12> r,
-                  VecP32q<12> x, const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
-  launch_cooperative(small_kernel(op, pl.wide), pl, st, FullSites<GeomBlk>{g}, op.U, p, t, r, x, size_t(0), a);
+cudaError_t launch_small(const WOp<float, G, VA, R1, LEAN>& op, const GeomBlk& g, VA<12> p, VA<12> t, VecP32q<12> r,
+                         VecP32q<12> x, const SmallArgs& a, const SmallPlan& pl, cudaStream_t st) {
+  return launch_cooperative(small_kernel(op, pl.wide), pl, st, FullSites<GeomBlk>{g}, op.U, p, t, r, x, size_t(0), a);
 }
 
 }  // namespace swc
