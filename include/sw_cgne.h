@@ -282,6 +282,8 @@ int sw_get_param(int key, double* value);
  * precision: SW_PREC_F32_RELIABLE or SW_PREC_F16_RELIABLE.  ms (HOST [3],
  * may be NULL) receives the times in ms, best (HOST, may be NULL) the chosen
  * width.  Allocates its own sources and solutions; blocks until done.
+ * On the small lattices of SW_PARAM_CHUNK, whose solves do not use the width,
+ * it is the kernels of larger lattices that are timed and set.
  * The width is process-wide: a system solved alone and in a batch is
  * bit-identical only under the same width, so tune before serving. */
 int sw_autotune(const sw_lattice* lat, int op, const void* U, const void* W, int nsys, int precision,

@@ -7,6 +7,8 @@
 // the fastest: sw_autotune over the register-blocking width NS in {1, 2, 4}
 // (SW_PARAM_NS_SW or SW_PARAM_NS_WILSON), sw_autotune_layout over width x site
 // order (SW_PARAM_SITE_BLOCKING: lexicographic or one of the site-block shapes).
+// On small lattices too they time the stencil kernels, which the settings are
+// for, and not the one-launch iterations, which ignore the width.
 #include <chrono>
 #include <vector>
 
@@ -45,6 +47,7 @@ double time_batch(const Geom& g, int op, const void* U, const void* W, int nsys,
     const auto t0 = std::chrono::steady_clock::now();
     SolveArgs a{static_cast<const double2*>(U), static_cast<const double2*>(W), chi.as<double2>(),
                 x.as<double2>(), nsys, masses.data(), r, 1e-30, iters, precision, nullptr, st};
+    a.one_launch = false;
     const int rc = op == SW_OP_WILSON ? wilson_cgne(g, a) : sw_cgne(g, a);
     const double t = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     if (rc < 0) return rc;

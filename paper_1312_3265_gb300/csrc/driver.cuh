@@ -350,9 +350,10 @@ class Engine {
   // a side stream and time launches with events when profiling is enabled;
   // all of these create driver resources, so allocation-free callers pass
   // false (they get one stream, direct launches and no timing samples).
+  // one_launch: small lattices may take the kernel of many iterations (small.cuh).
   Engine(const Geom& g, const OpD& opd, const OpF& opf, double r, int cap, double2* chi, double2* x,
          const Workspace& ws, SysState* hs_read, SysState* hs_stage, cudaStream_t st, cudaEvent_t ev,
-         bool use_graphs = true)
+         bool use_graphs = true, bool one_launch = true)
       : g_(g), opd_(opd), opf_(opf), r_(r), cap_(cap), chi_(chi), x_(x), ws_(ws), hr_(hs_read), hst_(hs_stage),
         st_(st), ev_(ev), n_((size_t)g.V * NC), s64_(n_ * f64_stride_factor<OpD>()),
         use_graphs_(use_graphs && param_graphs()),
@@ -382,7 +383,7 @@ class Engine {
     cls_ = ngrp_;
     set_grids(whole_, ngrp_);
     if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
-      small_ = small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
+      small_ = one_launch && small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
       if (small_) {
         for (int wide = 0; wide < (splan_.nt <= kSmallWide ? 2 : 1); ++wide) {
           int nb = 0;
@@ -1301,7 +1302,7 @@ int run_cgne_ws(const Geom& g, const OpD& opd, const OpF& opf, const SolveArgs& 
   using namespace std::chrono;
   const auto t0 = steady_clock::now();
   Engine<OpD, OpF, MIXED> e(g, opd, opf, a.r, a.nsys, const_cast<double2*>(a.chi), a.x, ws, hs, hs + a.nsys,
-                            a.stream, nullptr, use_graphs);
+                            a.stream, nullptr, use_graphs, a.one_launch);
   for (int i = 0; i < a.nsys; ++i)
     e.stage(i, a.masses[i], a.tols ? a.tols[i] : a.tol, a.max_iter, a.conv_b2 ? a.conv_b2[i] : 0.0);
   const long long max_rounds = 4LL * (a.max_iter / param_chunk() + 2) + 1000;

@@ -23,6 +23,7 @@ struct SolveArgs {
   sw_solve_info* infos;
   cudaStream_t stream;
   const double* tols = nullptr;  // host [nsys]: per-system tolerances (nullptr: tol for every system)
+  bool one_launch = true;  // small lattices: many iterations by one launch (false: always a launch per kernel)
   const double* conv_b2 = nullptr;  // host [nsys]: |b|^2 of an operator's own convergence criterion
 };
 
