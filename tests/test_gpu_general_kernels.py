@@ -30,14 +30,14 @@ class Batch:
         import torch
         g = torch.Generator("cuda").manual_seed(seed)
         V = ls.volume(dims)
-        # SU(3): unitary factor of a Gaussian near 1, its determinant's phase divided out
+        # SU(3) near 1: two rows by Gram-Schmidt, the third the conjugate of their cross product
         z = torch.eye(3, dtype=torch.complex128, device="cuda") + 0.3 * torch.randn(
-            (V * 4, 3, 3), dtype=torch.complex128, device="cuda", generator=g)
-        Q, R = torch.linalg.qr(z)
-        d = torch.diagonal(R, dim1=-2, dim2=-1)
-        Q = Q * (d / d.abs())[:, None, :]
+            (V, 4, 3, 3), dtype=torch.complex128, device="cuda", generator=g)
+        u = z[..., 0, :] / z[..., 0, :].norm(dim=-1, keepdim=True)
+        v = z[..., 1, :] - (z[..., 1, :] * u.conj()).sum(-1, keepdim=True) * u
+        v = v / v.norm(dim=-1, keepdim=True)
         self.sw, self.op, self.dims, self.apbc = sw, op, dims, apbc
-        self.U = (Q / torch.linalg.det(Q)[:, None, None] ** (1.0 / 3.0)).reshape(V, 4, 3, 3).contiguous()
+        self.U = torch.stack([u, v, torch.linalg.cross(u, v).conj()], dim=-2).contiguous()
         self.W = None
         if op == "sw":
             self.W = torch.empty((V, 8, 3, 3), dtype=torch.complex128, device="cuda")
@@ -100,3 +100,120 @@ def test_autotuners_time_the_kernels_they_tune(sw, op, prec):
         layout = sw.sw_kernel_launches() - before - one
     # three launches an iteration, two solves a candidate
     assert one >= 3 * 2 * 3 * iters and layout >= 3 * sw.SW_SITE_SHAPES * 2 * 3 * iters
+
+
+WILSON, SW, EO = (18, 14, 12, 10), (10, 12, 14, 10), (18, 16, 16, 14)  # 30240, 16800, 32256 sites (of a half)
+MASSES = [0.05, 0.1, 0.2, 0.07, 0.3, 0.02, 0.15]
+
+
+@pytest.mark.parametrize("op,dims", [("sw", SW), ("wilson", WILSON), ("wilson_eo", EO)])
+def test_widths_and_orders(sw, op, dims):
+    """Widths 1, 2 and 4 (7 systems: ragged groups) in two site orders and both
+    grid orders solve the same systems; the grid order does not change a bit."""
+    import torch
+    b = Batch(sw, op, dims, 7, 3, apbc=True)
+    for prec in ((1,) if op == "wilson_eo" else (1, 2)):
+        for width in (1, 2, 4):
+            for blocking in ((0,) if op == "wilson_eo" else (0, 1 + width)):
+                out = []
+                for gfast in (0, 1):
+                    with param(sw, NS_SW=width, NS_WILSON=width, SITE_BLOCKING=blocking, GROUP_FAST=gfast):
+                        x, infos, launches = b.solve(MASSES, prec)
+                    assert launches > 3 * max(i.iters for i in infos)
+                    out.append(x)
+                    for k in (0, 3, 6):
+                        assert b.residual(x, k, MASSES[k]) <= 1.01e-9
+                assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("op,dims,prec", [("sw", SW, 1), ("sw", SW, 2), ("wilson", WILSON, 1), ("wilson", WILSON, 2),
+                                          ("wilson_eo", EO, 1), ("sw", SW, 0), ("wilson", WILSON, 0)])
+def test_graphs_and_device_driven_rounds_are_bitwise_launches(sw, op, dims, prec):
+    """Chunks as graphs, updates on the side stream, and the whole solve as one
+    graph, on a stream that can be captured, against launches one by one."""
+    import torch
+    b = Batch(sw, op, dims, 3, 4, apbc=True)
+    masses = [0.05, 0.1, 0.2]
+    torch.cuda.synchronize()
+    ref = None
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for graphs, persistent in ((0, 0), (1, 0), (1, 1)):
+            with param(sw, GRAPHS=graphs, PERSISTENT=persistent):
+                x, infos, launches = b.solve(masses, prec)
+            torch.cuda.synchronize()
+            assert launches > 3 * max(i.iters for i in infos) > 3 * 16
+            got = [(i.iters, i.reliable_updates) for i in infos]
+            ref = (x, got) if ref is None else ref
+            assert got == ref[1] and torch.equal(x, ref[0])
+
+
+def test_wilson_lean_and_default_forms(sw):
+    import torch
+    b = Batch(sw, "wilson", WILSON, 5, 5, apbc=True)
+    out = []
+    for form in (0, 1):
+        with param(sw, WILSON_LEAN=form):
+            out.append(b.solve(MASSES[:5], 1))
+    assert [i.iters for i in out[0][1]] == [i.iters for i in out[1][1]]
+    assert torch.equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("op,dims,prec", [("sw", SW, 1), ("sw", SW, 2), ("wilson", WILSON, 1), ("wilson", WILSON, 2),
+                                          ("wilson_eo", EO, 1)])
+def test_other_wilson_parameters(sw, op, dims, prec):
+    b = Batch(sw, op, dims, 3, 6)
+    for r in (0.75, 1.3):
+        x, infos, launches = b.solve(MASSES[:3], prec, r=r)
+        assert launches > 3 * max(i.iters for i in infos)
+        for k in range(3):
+            assert b.residual(x, k, MASSES[k], r) <= 1.01e-9
+
+
+@pytest.mark.parametrize("op,dims,nsys,prec,r,kw", [
+    ("wilson", WILSON, 9, 1, 1.0, dict(NS_WILSON=4)), ("wilson", WILSON, 7, 1, 0.75, dict(NS_WILSON=2, GROUP_FAST=1)),
+    ("wilson", WILSON, 8, 2, 0.75, dict(SITE_BLOCKING=4)), ("wilson", WILSON, 9, 1, 1.0, dict(SITE_BLOCKING=2)),
+    ("sw", (18, 14, 16, 16), 13, 1, 1.0, dict(NS_SW=4)), ("sw", (18, 14, 16, 16), 13, 2, 1.3, dict(GROUP_FAST=1)),
+    ("sw", (18, 14, 16, 16), 12, 1, 0.75, dict(SITE_BLOCKING=5, NS_SW=1)), ("wilson_eo", EO, 7, 1, 0.75, {}),
+    ("wilson", WILSON, 3, 0, 0.75, {}), ("wilson_eo", EO, 3, 0, 1.0, {}), ("sw", SW, 5, 0, 1.3, {})])
+def test_halves_in_every_layout(sw, op, dims, nsys, prec, r, kw):
+    """Chunks as two halves: twice the launches, the same bits as every system alone."""
+    import torch
+    b = Batch(sw, op, dims, nsys, 8, apbc=True)
+    masses = [0.1 + 0.01 * (k % 5) for k in range(nsys)]
+    with param(sw, **kw), torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda.synchronize()
+        x, infos, launches = b.solve(masses, prec, r=r)
+        assert launches > 5 * max(i.iters for i in infos)
+        for k, m in enumerate(masses):
+            one = torch.zeros_like(b.chi[k])
+            info = sw.cgne_solve(dims, OPS[op], b.U, b.W, b.chi[k].contiguous(), one, m, r, 1e-9, 5000, prec, True)
+            assert info.iters == infos[k].iters and torch.equal(one, x[k])
+        torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("op,dims,prec", [("sw", SW, 1), ("wilson", WILSON, 1), ("wilson", WILSON, 2),
+                                          ("sw", SW, 0)])
+def test_server_engines(sw, op, dims, prec):
+    """Requests that join while others run, more of them than slots, against single solves."""
+    import torch
+    n = 9
+    b = Batch(sw, op, dims, n, 9, apbc=True)
+    torch.cuda.synchronize()  # the engine copies U on a stream of its own
+    srv = sw.Server(8 << 30)
+    try:
+        e = srv.add_engine(dims, OPS[op], b.U, precision=prec, slots=5, t_antiperiodic=True)
+        chi = b.chi.cpu().pin_memory()
+        x = torch.zeros_like(chi).pin_memory()
+        masses = [0.05 + 0.03 * ((5 * k) % n) for k in range(n)]
+        ids = {srv.submit(e, chi[k], x[k], m, 1e-9): k for k, m in enumerate(masses)}
+        srv.drain(120)
+        done = srv.poll()
+        assert len(done) == n
+        for rid, info in done:
+            k = ids[rid]
+            one = torch.zeros_like(b.chi[k])
+            ref = sw.cgne_solve(dims, OPS[op], b.U, b.W, b.chi[k].contiguous(), one, masses[k], 1.0, 1e-9, 100000,
+                                prec, True)
+            assert info.iters == ref.iters and torch.equal(one.cpu(), x[k])
+    finally:
+        srv.close()
