@@ -211,7 +211,8 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  *   system whose reliable update ran beside a chunk resumes with the next one.
  *   Mixed-precision solves on lattices that a few hundred warps hold (at 152
  *   SMs: Wilson up to 29184 sites, even-odd twice that, staggered Wilson
- *   14592) run up to 512 iterations in one launch instead.
+ *   14592) run up to 512 iterations in one launch instead (a server's engine 32
+ *   or more, by how many systems share the blocks).
  * SW_PARAM_RELIABLE_DELTA: mixed precision only; the FP32 correction is
  *   folded into the FP64 solution and r = b - A x recomputed in FP64 when the
  *   iterated |r| falls below delta times its maximum since the last such

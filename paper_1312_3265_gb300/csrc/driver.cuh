@@ -81,6 +81,19 @@ constexpr int kOver64 = 8;  // waves of blocks of the FP64 kernels
 // 3.93 / 3.82; 16^4, 3: 35.9 / 33.9; even-odd 8^3x16, 12: 24.6 / 21.8.
 constexpr double kSplitWork = 1 << 21, kSplitGauge = 80e6, kSplitWork64 = 1 << 14;
 
+// Whether an engine takes the one-launch iterations on small lattices: never (the
+// autotuners'), as a solve, or as a server, whose requests arrive while it runs
+// and whose freed slots wait for the launch's end.  A server's launch is bounded
+// to about a millisecond: kSmallIters iterations over the systems of a group, at
+// least kServeIters.  Launches of kSmallIters against this bound: 40 long Wilson
+// solves on 12^4 keep a short request waiting for 0.46 / less than 0.25 of their
+// time; 48 slots on 6x10x12x14, always full, 1407-1447 / 1456-1500 requests/s, at
+// 1078 requests/s a mean latency of 15.4-18.1 / 14.1-15.0 ms; the same where groups
+// hold few systems.  A bound of kServeIters for every group loses where systems
+// have groups of their own (4^3x8, 24 slots: 5053 / 4219 requests/s).
+enum class OneLaunch { kNever, kSolve, kServe };
+constexpr int kServeIters = 32;
+
 // over: waves of blocks at most.  Kernels bound by the FP64 pipe take several:
 // blocks that share the pipe do not run in rounds, and a block that loops over
 // tiles would leave the last of them to a few SMs (8^3x16, 12 systems: 256
@@ -350,13 +363,13 @@ class Engine {
   // a side stream and time launches with events when profiling is enabled;
   // all of these create driver resources, so allocation-free callers pass
   // false (they get one stream, direct launches and no timing samples).
-  // one_launch: small lattices may take the kernel of many iterations (small.cuh).
+  // one_launch: use of the kernel of many iterations (small.cuh) on small lattices.
   Engine(const Geom& g, const OpD& opd, const OpF& opf, double r, int cap, double2* chi, double2* x,
          const Workspace& ws, SysState* hs_read, SysState* hs_stage, cudaStream_t st, cudaEvent_t ev,
-         bool use_graphs = true, bool one_launch = true)
+         bool use_graphs = true, OneLaunch one_launch = OneLaunch::kSolve)
       : g_(g), opd_(opd), opf_(opf), r_(r), cap_(cap), chi_(chi), x_(x), ws_(ws), hr_(hs_read), hst_(hs_stage),
         st_(st), ev_(ev), n_((size_t)g.V * NC), s64_(n_ * f64_stride_factor<OpD>()),
-        use_graphs_(use_graphs && param_graphs()),
+        one_launch_(one_launch), use_graphs_(use_graphs && param_graphs()),
         driver_resources_(use_graphs) {
     ntiles_ = (g.V + kTile - 1) / kTile;
     pstride_ = kWarps * ntiles_;
@@ -383,7 +396,7 @@ class Engine {
     cls_ = ngrp_;
     set_grids(whole_, ngrp_);
     if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
-      small_ = one_launch && small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
+      small_ = one_launch != OneLaunch::kNever && small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
       if (small_) {
         for (int wide = 0; wide < (splan_.nt <= kSmallWide ? 2 : 1); ++wide) {
           int nb = 0;
@@ -929,6 +942,9 @@ class Engine {
       splan_.wide = small_blocks_[1] >= units * splan_.tiles;
       splan_.groups = std::max(1, std::min(units, small_blocks_[splan_.wide] / splan_.tiles));
       splan_.windows = (bound * per + splan_.groups * kSmallShare - 1) / (splan_.groups * kSmallShare);
+      // (systems a group of blocks holds)
+      const int share = per * ((units + splan_.groups * splan_.windows - 1) / (splan_.groups * splan_.windows));
+      const int iters = one_launch_ == OneLaunch::kServe ? std::max(kServeIters, kSmallIters / share) : kSmallIters;
       unsigned* bad = reinterpret_cast<unsigned*>(ws_.list + cap_ + 1);
       if (small_epochs_.restart()) clear_small();
       build_list<<<1, 256, 0, st_>>>(cap_, ws_.S, ws_.list, bad, splan_.groups, per);
@@ -936,7 +952,7 @@ class Engine {
         const cudaError_t e =
             launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
                          SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epochs_.take(),
-                                   w, splan_.windows, polls_},
+                                   w, splan_.windows, polls_, iters},
                          splan_, st_);
         launches(w ? 1 : 2);
         if (e != cudaSuccess) {
@@ -1253,6 +1269,7 @@ class Engine {
   SmallPlan splan_;
   int small_blocks_[2] = {0, 0};  // blocks of its two forms resident at once
   BarrierEpochs small_epochs_;
+  OneLaunch one_launch_;
   int polls_ = 1;
   std::vector<Sample> samples_;
   std::vector<FpSample> fsamples_;
@@ -1302,7 +1319,7 @@ int run_cgne_ws(const Geom& g, const OpD& opd, const OpF& opf, const SolveArgs& 
   using namespace std::chrono;
   const auto t0 = steady_clock::now();
   Engine<OpD, OpF, MIXED> e(g, opd, opf, a.r, a.nsys, const_cast<double2*>(a.chi), a.x, ws, hs, hs + a.nsys,
-                            a.stream, nullptr, use_graphs, a.one_launch);
+                            a.stream, nullptr, use_graphs, a.one_launch ? OneLaunch::kSolve : OneLaunch::kNever);
   for (int i = 0; i < a.nsys; ++i)
     e.stage(i, a.masses[i], a.tols ? a.tols[i] : a.tol, a.max_iter, a.conv_b2 ? a.conv_b2[i] : 0.0);
   const long long max_rounds = 4LL * (a.max_iter / param_chunk() + 2) + 1000;

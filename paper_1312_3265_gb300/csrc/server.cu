@@ -136,7 +136,7 @@ static int build_engine(const Geom& g, int cap, double r, int prec, MakeOps make
   if (cudaMallocHost((void**)&impl->hs, sizeof(SysState) * 2 * cap) != cudaSuccess) return SW_ERR_OOM;
   const Workspace ws = carve_workspace_for<typename OpF::Vec>(wsm, g.V, OpD::NC, cap, MIXED);
   impl->e = std::make_unique<Engine<OpD, OpF, MIXED>>(g, opd, opf, r, cap, chi, x, ws, impl->hs, impl->hs + cap,
-                                                      impl->st, impl->ev);
+                                                      impl->st, impl->ev, true, OneLaunch::kServe);
   if (const cudaError_t e = cudaStreamSynchronize(impl->st); e != cudaSuccess) return cuda_fail(e);
   *out = std::move(impl);
   return SW_OK;

@@ -105,6 +105,7 @@ struct SmallArgs {
   unsigned epoch;             // above every epoch of the launches before
   int window, windows;        // this launch's part of the list
   int polls;                  // polls after which a wait gives up
+  int iters;                  // iterations at most
 };
 
 // ---------------------------------------------------------------- the group's state and barriers
@@ -571,7 +572,7 @@ __global__ void __launch_bounds__(MAXT, 1)
   };
   if constexpr (!kEO) load_links(0);
   bool ok = true;
-  for (int it = 0; it < kSmallIters; ++it) {
+  for (int it = 0; it < a.iters; ++it) {
     if constexpr (kEO)
       if (!(ok = odd_pass(p, false))) break;
 #pragma unroll 1
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(MAXT, 1)
   };
   unsigned epoch = a.epoch;
   bool ok = true;
-  for (int it = 0; it < kSmallIters; ++it) {
+  for (int it = 0; it < a.iters; ++it) {
 #pragma unroll 1
     for (int k = 0; k < share; k += 2) {
       const int mask = s.on[k] | (s.on[k + 1] << 1);
