@@ -347,15 +347,12 @@ __device__ __forceinline__ void site_results(const Op& op, const GG& g, int n, c
 // ---------------------------------------------------------------- plain apply (ABI)
 // out = (D+m) in, or (D+m)^+ in with dagger; with has_sub, out = sub - (D+m) in
 // (the FP64 residual chi - (D+m) x of a reliable update).
-// Blocks per SM of the one-thread-a-site FP64 kernels: the spin-projected Wilson
-// operator at 128 registers (4 blocks) instead of 138 (3): 214 against 219 us at
-// 16^3x32, 1040 against 1064 at 24^3x48; the others fit 3 blocks (168).
-template <class Op> struct fp64_blocks : std::integral_constant<int, 3> {};
-template <typename G, template <int> class VA> struct fp64_blocks<WOp<double, G, VA, true, false>>
-    : std::integral_constant<int, 4> {};
-
+// 3 blocks per SM: the spin-projected Wilson operator takes 138 registers.  Held
+// to 128 for 4 blocks it spills, and is no faster: 16^3x32 213.4 us against 213.1,
+// 24^3x48 1047.6-1048.9 against 1045.8-1046.1; on fields not touched before
+// (16^3x32) 248 against 246.5.
 template <typename T, typename Op>
-__global__ void __launch_bounds__(kTile, fp64_blocks<Op>::value) apply_kernel(Geom g, Op op, typename Op::Vec in, typename Op::Vec out,
+__global__ void __launch_bounds__(kTile, 3) apply_kernel(Geom g, Op op, typename Op::Vec in, typename Op::Vec out,
                                                     double mass0, size_t sstride, double r, int dagger,
                                                     const SysState* S, int only_status, int* nact = nullptr,
                                                     typename Op::Vec sub = {}, int has_sub = 0) {
