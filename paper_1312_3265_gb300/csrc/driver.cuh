@@ -260,7 +260,7 @@ inline size_t workspace_bytes_pt(int V, int NC, int nsys, bool mixed, size_t pt,
   b += mixed ? 2 * align_up(pt * nsys_pt) + 2 * align_up(sizeof(float2) * n32) : align_up(pt * nsys_pt);
   b += align_up(sizeof(SysState) * nsys) + align_up(sizeof(double) * 2 * kWarps * ntiles * nsys) +
        align_up(sizeof(unsigned) * 2 * nsys) + align_up(sizeof(double) * nsys) +
-       (mixed ? align_up(8 * small_slots(V, nsys)) + align_up(sizeof(int) * small_words(V, nsys)) : 0) +
+       (mixed ? align_up(8 * small_slots(V, NC, nsys)) + align_up(sizeof(int) * small_words(V, NC, nsys)) : 0) +
        align_up(sizeof(double) * 2 * kHist * nsys) + align_up(sizeof(int) * 2 * kProfSlots) +
        align_up(sizeof(int) * 8);
   return b;
@@ -307,8 +307,8 @@ inline Workspace carve_workspace_pt(void* base, int V, int NC, int nsys, bool mi
   w.tickets = (unsigned*)take(sizeof(unsigned) * 2 * nsys);  // 2nd half: the reliable-update kernels
   w.mass = (double*)take(sizeof(double) * nsys);
   if (mixed) {
-    w.slots = (unsigned long long*)take(8 * small_slots(V, nsys));
-    w.list = (int*)take(sizeof(int) * small_words(V, nsys));
+    w.slots = (unsigned long long*)take(8 * small_slots(V, NC, nsys));
+    w.list = (int*)take(sizeof(int) * small_words(V, NC, nsys));
   }
   w.hist = (double*)take(sizeof(double) * 2 * kHist * nsys);
   w.pcount = (int*)take(sizeof(int) * 2 * kProfSlots);
@@ -396,6 +396,7 @@ class Engine {
     cls_ = ngrp_;
     set_grids(whole_, ngrp_);
     if constexpr (MIXED && small_traits<OpF>::kSites > 0) {
+      static_assert(small_traits<OpF>::kSites == small_sites(NC), "the workspace's plan");
       small_ = one_launch != OneLaunch::kNever && small_tiles(g.V, small_traits<OpF>::kSites, &splan_);
       if (small_) {
         for (int wide = 0; wide < (splan_.nt <= kSmallWide ? 2 : 1); ++wide) {
@@ -926,8 +927,8 @@ class Engine {
 
   // The small-lattice kernels' list, "gave up" words and inboxes, zeroed.
   void clear_small() {
-    cudaMemsetAsync(ws_.slots, 0, 8 * small_slots(g_.V, cap_), st_);
-    cudaMemsetAsync(ws_.list, 0, sizeof(int) * small_words(g_.V, cap_), st_);
+    cudaMemsetAsync(ws_.slots, 0, 8 * small_slots(g_.V, NC, cap_), st_);
+    cudaMemsetAsync(ws_.list, 0, sizeof(int) * small_words(g_.V, NC, cap_), st_);
   }
 
   // Small lattices: many iterations of every running system by one launch (a
@@ -940,7 +941,8 @@ class Engine {
       // the form with every load under way where each system has blocks of its
       // own, else the one of which more blocks are resident
       splan_.wide = small_blocks_[1] >= units * splan_.tiles;
-      splan_.groups = std::max(1, std::min(units, small_blocks_[splan_.wide] / splan_.tiles));
+      splan_.groups = std::max(1, std::min({units, small_blocks_[splan_.wide] / splan_.tiles,
+                                            small_groups(splan_.tiles)}));
       splan_.windows = (bound * per + splan_.groups * kSmallShare - 1) / (splan_.groups * kSmallShare);
       // (systems a group of blocks holds)
       const int share = per * ((units + splan_.groups * splan_.windows - 1) / (splan_.groups * splan_.windows));
@@ -951,7 +953,8 @@ class Engine {
       for (int w = 0; w < splan_.windows; ++w) {
         const cudaError_t e =
             launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
-                         SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots, bad + cap_, bad, small_epochs_.take(),
+                         SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots,
+                                   small_boxes(splan_.tiles, cap_), bad + cap_, bad, small_epochs_.take(),
                                    w, splan_.windows, polls_, iters},
                          splan_, st_);
         launches(w ? 1 : 2);

@@ -101,7 +101,8 @@ struct SmallArgs {
   RedBuf rb;
   BatchParams bp;
   int nsys;
-  unsigned long long* slots;  // [2][nsys][tiles][tiles][2] each block's inbox: tagged halves of the tile sums
+  unsigned long long* slots;  // [2][boxes][tiles][tiles][2] each block's inbox: tagged halves of the tile sums
+  int boxes;                  // nsys, or kSmallShare a group where that is less
   unsigned* flags;            // [groups][tiles][tiles] each block's inbox: barrier epochs
   unsigned* bad;              // [groups] "gave up"
   unsigned epoch;             // above every epoch of the launches before
@@ -182,13 +183,18 @@ __device__ __forceinline__ bool group_barrier(const SmallArgs& a, SmallShared& s
 // each block moves its copy of the states on (block 0 records the
 // coefficients).  The slots of a phase are written again only after every block
 // has passed a later barrier.
+// The slots of system t of the group: by its number in the batch, or by the
+// group's t where the batch takes several launches (whose words the epochs tell apart).
+__device__ __forceinline__ size_t box(const SmallArgs& a, const SmallShared& s, int t) {
+  return a.boxes < a.nsys ? blockIdx.y * kSmallShare + t : s.sys[t];
+}
 template <int PHASE>
 __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int share, unsigned& epoch) {
   ++epoch;
   __syncthreads();
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, nt = gridDim.x;
   const unsigned long long tag = (unsigned long long)epoch << 32;
-  unsigned long long* slots = a.slots + (size_t)(PHASE - 1) * a.nsys * nt * nt * 2;
+  unsigned long long* slots = a.slots + (size_t)(PHASE - 1) * a.boxes * nt * nt * 2;
   // The block's stores, before any of its words: by every warp that may post
   // one, whichever of its systems still run.
   if ((int)(threadIdx.x >> 5) < share) fence_gpu();
@@ -197,12 +203,12 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
     double v = s.wsum[t][0];
     for (int w = 1; w < nw; ++w) v += s.wsum[t][w];
     const unsigned long long hi = tag | (unsigned)__double2hiint(v), lo = tag | (unsigned)__double2loint(v);
-    for (int i = lane; i < nt; i += 32) st_relaxed(slots + (((size_t)s.sys[t] * nt + i) * nt + blockIdx.x) * 2, hi, lo);
+    for (int i = lane; i < nt; i += 32) st_relaxed(slots + ((box(a, s, t) * nt + i) * nt + blockIdx.x) * 2, hi, lo);
   }
   int n = 0;
   for (int t = threadIdx.x >> 5; t < share; t += nw) {
     if (!s.on[t]) continue;
-    const unsigned long long* p = slots + ((size_t)s.sys[t] * nt + blockIdx.x) * nt * 2;
+    const unsigned long long* p = slots + (box(a, s, t) * nt + blockIdx.x) * nt * 2;
     double v = 0.0;
     for (int i0 = lane; i0 < nt; i0 += 32 * kPolls) {
       unsigned long long hi[kPolls], lo[kPolls];
@@ -915,18 +921,6 @@ struct SmallPlan {
   bool wide = false;
 };
 
-// Tiles a small lattice can have (0: too large for any operator), for the
-// workspace: its blocks hold at least 32 sites and are at most one per SM.
-inline size_t small_tiles_bound(int V) {
-  return V > sm_count() * kSmallThreads / 2 ? 0 : std::min<size_t>(sm_count(), ((size_t)V + 31) / 32);
-}
-inline size_t small_slots(int V, int nsys) {  // 64-bit words of the inboxes
-  return 4 * small_tiles_bound(V) * small_tiles_bound(V) * nsys;
-}
-inline size_t small_words(int V, int nsys) {  // ints: list, "gave up" words, barrier epochs
-  return small_tiles_bound(V) ? 1 + 2 * (size_t)nsys + small_tiles_bound(V) * small_tiles_bound(V) * nsys : 0;
-}
-
 // Whether a lattice of V sites (of the operator's vectors) takes the small
 // form, and its blocks: as few warps a block as spread the lattice over every
 // SM.  By the volume only.
@@ -939,6 +933,25 @@ inline bool small_tiles(int V, int sites_per_warp, SmallPlan* p) {
   p->nt = 32 * per;
   p->tiles = (int)((warps + per - 1) / per);
   return true;
+}
+
+// Scratch of a batch of nsys systems of NC components on V sites: the inboxes'
+// 64-bit words, and the ints of the list, the "gave up" words and the barrier
+// epochs (0: the lattice does not take the small form).  Bounded by the groups
+// resident at once (at most two blocks an SM), so that the workspace of a large
+// batch grows by little (8^4 staggered Wilson, 600 systems: 46 MB on 480).
+constexpr int small_sites(int NC) { return NC == 3 ? 8 : 16; }  // a warp holds
+inline int small_groups(int tiles) { return std::max(1, 2 * sm_count() / tiles); }
+inline int small_boxes(int tiles, int nsys) { return std::min(nsys, small_groups(tiles) * kSmallShare); }
+inline size_t small_slots(int V, int NC, int nsys) {
+  SmallPlan p;
+  if (!small_tiles(V, small_sites(NC), &p)) return 0;
+  return (size_t)4 * p.tiles * p.tiles * small_boxes(p.tiles, nsys);
+}
+inline size_t small_words(int V, int NC, int nsys) {
+  SmallPlan p;
+  if (!small_tiles(V, small_sites(NC), &p)) return 0;
+  return 1 + 2 * (size_t)nsys + (size_t)p.tiles * p.tiles * std::min(nsys, small_groups(p.tiles));
 }
 
 // Refused (an error returned, nothing launched) where the grid cannot be

@@ -140,3 +140,27 @@ def test_a_wait_that_gives_up_is_a_timeout(sw, op, prec):
     x = torch.zeros_like(chi)
     rc, infos = solve(x)
     assert rc == sw.SW_OK and all(i.true_rel_resid <= 1e-9 for i in infos)
+
+
+@pytest.mark.parametrize("op,dims,nsys,base", [("sw", (8, 8, 8, 8), 600, 3 * 64), ("wilson", (12, 12, 12, 16), 90, 12 * 64)])
+def test_scratch_of_a_large_batch_stays_small(sw, op, dims, nsys, base):
+    """The workspace of a batch on a small lattice is that of larger lattices (two
+    FP64 vectors, p, t, r and x: `base` bytes a site and system, and the packed
+    gauge field) and at most a fifth of it."""
+    import torch
+    g = torch.Generator("cuda").manual_seed(1)
+    V = ls.volume(dims)
+    U = su3_field(V, g)
+    W = None
+    if op == "sw":
+        W = torch.empty((V, 8, 3, 3), dtype=torch.complex128, device="cuda")
+        sw.sw_hypercube_build(dims, U, W, False)
+    chi = torch.randn((nsys, V) + ((3,) if op == "sw" else (4, 3)), dtype=torch.complex128, device="cuda", generator=g)
+    x = torch.zeros_like(chi)
+    torch.cuda.synchronize()
+    sw.sw_trim_workspace()
+    held = sw.sw_workspace_reserved()
+    rc, infos = sw.cgne_solve_batch(dims, OPS[op], U, W, chi, x, [0.5] * nsys, 1.0, 1e-6, 5000, 1, False)
+    assert rc == sw.SW_OK and all(i.true_rel_resid <= 1e-6 for i in infos)
+    used = sw.sw_workspace_reserved() - held
+    assert used <= 1.2 * (base * V * nsys + 864 * V) + (32 << 20)  # (and the pool's granularity)
