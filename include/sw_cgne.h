@@ -208,7 +208,8 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  * SW_PARAM_CHUNK: CG iterations launched between two reads of the per-system
  *   status words (1..4096, default 4).  Larger chunks mean fewer host
  *   synchronisations; converged systems idle for at most one chunk, and a
- *   system whose reliable update ran beside a chunk resumes with the next one.
+ *   system whose reliable update ran beside a chunk resumes within it, at every
+ *   fourth iteration.
  *   Mixed-precision solves on lattices that a few hundred warps hold (at 152
  *   SMs: Wilson up to 29184 sites, even-odd twice that, staggered Wilson
  *   14592) run up to 512 iterations in one launch instead (a server's engine 32

@@ -708,8 +708,8 @@ __global__ void __launch_bounds__(256) cg_k3_pair(int V, RVec r, PVec p, RVec x,
 // ST_NEED_RU by the host's round, so that iterations running at the same time
 // on another stream -- which may move other systems to ST_NEED_RU -- cannot
 // change the set while the update's kernels run).  It ends in ST_READY;
-// commit_ready, launched on the iteration stream at the start of a chunk, lets
-// the system run again.
+// commit_ready, launched on the iteration stream at the start of a chunk and
+// within it, lets the system run again.
 // r64 = (D+m)^+ t64 with t64 = chi - (D+m) x (apply_kernel's has_sub form), so
 // r64 = b - A x for b = (D+m)^+ chi; |r64|^2, then the convergence decision.
 // An operator with a full-system criterion (full_conv) also sums its

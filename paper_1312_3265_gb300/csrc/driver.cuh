@@ -65,6 +65,10 @@ template <class Op> bool use_quad(int V) {
   if constexpr (has_quad<Op>()) return V <= Op::kQuadVolume;
   return false;
 }
+// Iterations of a chunk between two looks for systems whose reliable update has
+// ended beside it (a launch each): the default chunk, so that in a longer one
+// (SW_PARAM_CHUNK) they need not wait for its end.
+constexpr int kCommitEvery = 4;
 constexpr int kOver64 = 8;  // waves of blocks of the FP64 kernels
 // A chunk runs as two halves (Engine::run_chunk) from this many complex numbers in
 // a vector of the running systems (below, a half's launches are as short as the
@@ -734,13 +738,15 @@ class Engine {
           cudaStreamWaitEvent(side_, ev_fork_, 0);
           reliable_update(cap_, side_);
           cudaEventRecord(ev_join_, side_);
-          commit(whole_, body_st);
-          for (int i = 0; i < chunk_; ++i) iterate(whole_, body_st, false, false);
+          for (int i = 0; i < chunk_; ++i) {
+            if (i % kCommitEvery == 0) commit(whole_, body_st);
+            iterate(whole_, body_st, false, false);
+          }
           cudaStreamWaitEvent(body_st, ev_join_, 0);
           round_end<<<1, 256, 0, body_st>>>(cap_, S, ws_.ctl, max_rounds, loop);
           cudaGraph_t body = nullptr;
           ok = cudaStreamEndCapture(body_st, &body) == cudaSuccess;
-          per_round = 3 + (MIXED ? 7 : 5) + 3 * chunk_ + (two_pass<OpF>::value ? 2 * chunk_ + 2 : 0);
+          per_round = 2 + commits() + (MIXED ? 7 : 5) + 3 * chunk_ + (two_pass<OpF>::value ? 2 * chunk_ + 2 : 0);
         }
       }
       ok = ok && cudaStreamUpdateCaptureDependencies(st_, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies) ==
@@ -1002,7 +1008,7 @@ class Engine {
     }
     if (ge) {
       cudaGraphLaunch(ge, st_);
-      launches((split_ ? 2 : 1) * (1 + 3 * chunk_));
+      launches((split_ ? 2 : 1) * (commits() + 3 * chunk_));
       if (prof()) {
         prof_count(cls_k1(), chunk_);
         prof_count(cls_k2(), chunk_);
@@ -1018,7 +1024,8 @@ class Engine {
     int s0 = 0, n = 0, ngrp = 0, g1 = 0, g2 = 0, gV = 0;
   };
 
-  // READY -> RUNNING, at a chunk's start.
+  // READY -> RUNNING, at a chunk's start and every kCommitEvery iterations of it.
+  int commits() const { return (chunk_ + kCommitEvery - 1) / kCommitEvery; }
   void commit(const Range& q, cudaStream_t s) { commit_ready<<<(q.n + 127) / 128, 128, 0, s>>>(q.n, ws_.S + q.s0); }
 
   // A chunk of iterations on the engine's stream -- or as two halves of the
@@ -1030,19 +1037,23 @@ class Engine {
     if (split_ && !sample) {
       cudaEventRecord(ev_split_, st_);
       cudaStreamWaitEvent(half_st_, ev_split_, 0);
-      commit(half_[0], st_);
-      commit(half_[1], half_st_);
       for (int i = 0; i < chunk_; ++i) {
+        if (i % kCommitEvery == 0) {
+          commit(half_[0], st_);
+          commit(half_[1], half_st_);
+        }
         iterate(half_[0], st_, false, count);
         iterate(half_[1], half_st_, false, count);
       }
       cudaEventRecord(ev_meet_, half_st_);
       cudaStreamWaitEvent(st_, ev_meet_, 0);
-      if (count) launches(2);
+      if (count) launches(2 * commits());
     } else {
-      commit(whole_, st_);
-      for (int i = 0; i < chunk_; ++i) iterate(whole_, st_, sample && i == 1, count);
-      if (count) launches(1);
+      for (int i = 0; i < chunk_; ++i) {
+        if (i % kCommitEvery == 0) commit(whole_, st_);
+        iterate(whole_, st_, sample && i == 1, count);
+      }
+      if (count) launches(commits());
     }
   }
 

@@ -260,12 +260,11 @@ static __global__ void mark_ready(int nsys, SysState* S) {
   if (i < nsys && S[i].status == ST_JUST_UPDATED) S[i].status = ST_READY;
 }
 
-// First launch of a chunk of CG iterations, on the iteration stream: READY ->
-// RUNNING.  A reliable update running concurrently on another stream marks
+// First launch of a chunk of CG iterations and of every fourth of its iterations,
+// on the iteration stream: READY -> RUNNING.  A reliable update running concurrently on another stream marks
 // its systems READY only after all its writes (x, r, p) are complete, and the
-// switch happens between chunks, so every kernel of an iteration sees the
-// same set of running systems.  (As the first launch of every iteration it cost
-// a launch each; a system waits at most a chunk, as it does for its update.)
+// switch happens between iterations, so every kernel of an iteration sees the
+// same set of running systems.  (Before every iteration it cost a launch each.)
 static __global__ void commit_ready(int nsys, SysState* S) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nsys && S[i].status == ST_READY) S[i].status = ST_RUNNING;

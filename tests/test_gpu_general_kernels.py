@@ -217,3 +217,25 @@ def test_server_engines(sw, op, dims, prec):
             assert info.iters == ref.iters and torch.equal(one.cpu(), x[k])
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("persistent", [0, 1])
+def test_a_system_resumes_within_a_long_chunk(sw, persistent):
+    """Two systems, chunks of 64 iterations: the heavy one's update runs beside the
+    second chunk, in which it goes on to its end, while the light one runs to its
+    iteration limit of 128.  Two chunks, then, and on the device a third round for
+    the last updates; a system that resumed only with the next chunk takes one more."""
+    import torch
+    b = Batch(sw, "wilson", WILSON, 2, 3)
+    V = ls.volume(WILSON)
+    b.U = torch.eye(3, dtype=torch.complex128, device="cuda").expand(V, 4, 3, 3).contiguous()  # free: slow at mass 0.01
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()), param(sw, CHUNK=64, PERSISTENT=persistent):
+        x = torch.zeros_like(b.chi)
+        before = sw.sw_kernel_launches()
+        rc, infos = sw.cgne_solve_batch(b.dims, 1, b.U, None, b.chi, x, [6.0, 0.01], 1.0, 1e-10, 128, 1)
+        launches = sw.sw_kernel_launches() - before
+        torch.cuda.synchronize()
+    assert infos[0].status == sw.SW_OK and infos[0].iters < 40
+    assert infos[1].status == sw.SW_NOT_CONVERGED and infos[1].iters == 128
+    assert launches < 3.9 * 64 * 3
