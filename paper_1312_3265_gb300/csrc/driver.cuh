@@ -950,6 +950,7 @@ class Engine {
       splan_.groups = std::max(1, std::min({units, small_blocks_[splan_.wide] / splan_.tiles,
                                             small_groups(splan_.tiles)}));
       splan_.windows = (bound * per + splan_.groups * kSmallShare - 1) / (splan_.groups * kSmallShare);
+      const int fetch = 4.0 * sizeof(float2) * NC * g_.V * live_slots() > kSmallFetch;
       // (systems a group of blocks holds)
       const int share = per * ((units + splan_.groups * splan_.windows - 1) / (splan_.groups * splan_.windows));
       const int iters = one_launch_ == OneLaunch::kServe ? std::max(kServeIters, kSmallIters / share) : kSmallIters;
@@ -961,7 +962,7 @@ class Engine {
             launch_small(opf_, gb_, fp_, ft_, fr_, fx_,
                          SmallArgs{ws_.list, ws_.S, rb_, bp_, cap_, ws_.slots,
                                    small_boxes(splan_.tiles, cap_), bad + cap_, bad, small_epochs_.take(),
-                                   w, splan_.windows, polls_, iters},
+                                   w, splan_.windows, polls_, iters, fetch},
                          splan_, st_);
         launches(w ? 1 : 2);
         if (e != cudaSuccess) {

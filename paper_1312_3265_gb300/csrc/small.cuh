@@ -57,6 +57,7 @@ constexpr int kSmallWide = 256;     // largest block of the 255-register form
 // room of the inboxes.
 constexpr int kSmallWarps = 6;
 constexpr int kSmallShare = 64;     // systems a group of blocks holds
+constexpr double kSmallFetch = 1 << 27;  // bytes of the running systems' vectors from which they are fetched ahead
 constexpr int kSmallIters = 512;    // iterations a launch at most
 static_assert(5 * kSmallIters < BarrierEpochs::kLaunch, "epochs of a launch (even-odd: 5 an iteration)");
 
@@ -109,6 +110,7 @@ struct SmallArgs {
   int window, windows;        // this launch's part of the list
   int polls;                  // polls after which a wait gives up
   int iters;                  // iterations at most
+  int fetch;                  // the vectors of the running systems exceed L2: prefetch the next system's
 };
 
 // ---------------------------------------------------------------- the group's state and barriers
@@ -353,6 +355,10 @@ __device__ __forceinline__ void flush_norms(NormBuf<NV>& b, SmallShared& sh, int
 // launch's phases).
 template <class V> struct SpinorIO;
 template <> struct SpinorIO<VecP32q<12>> {
+  // a warp's 16 sites from n0 (12 lines) into L2
+  __device__ static __forceinline__ void prefetch(const VecP32q<12>& v, int n0, int lane) {
+    if (lane < 12) asm volatile("prefetch.global.L2 [%0];" ::"l"(v.p + pk(n0, 6, 0) + lane * 8));
+  }
   struct Raw { float4 q[6]; };
   __device__ static __forceinline__ unsigned offset(int n) { return (unsigned)pk(n, 6, 0); }
   __device__ static __forceinline__ Raw load(const VecP32q<12>& v, unsigned off, int) {
@@ -559,6 +565,20 @@ __global__ void __launch_bounds__(MAXT, 1)
     v.p += scratch;
     return v;
   };
+  // The system after k whose lines are to be fetched ahead (-1: none).  A system's
+  // turn in a phase is latency, of which its own and its neighbours' first loads
+  // from memory are the most where the batch's vectors exceed L2; each block
+  // fetches its own sites.  FP32 spinors from kSmallFetch bytes of p, t, r and x, a
+  // solve to 1e-8 of 48 systems, without / with: 6x10x12x14 27.2 / 26.6 ms, 12^4
+  // 46.1 / 43.7, 12^3x16 56.7 / 53.3; below, 8^4 13.2 / 13.5, 12^3x16 with 12
+  // systems 15.75 / 15.79.  FP16 storage (half the bytes) and the even-odd
+  // operator (its scratch is read, too) gain less than they lose: 36.2 / 37.8 and
+  // 61.6 / 62.5.
+  constexpr bool kFetch = !kEO && std::is_same<VI, VecP32q<12>>::value;
+  const int n0 = nn - (lane & 15);
+  auto next = [&](int k) {
+    return kFetch && a.fetch && k + 1 < share && n0 < V && s.on[k + 1] ? s.sys[k + 1] : -1;
+  };
   unsigned epoch = a.epoch;
   // even-odd: u = D_oe v of every running system into v's scratch
   auto odd_pass = [&](const VI& v, bool dagger) {
@@ -586,6 +606,8 @@ __global__ void __launch_bounds__(MAXT, 1)
       if (s.on[k]) {
         const VI w = sys_view(p, s.sys[k], a.bp.vstride);
         float o[12], own[12];
+        if constexpr (kFetch)
+          if (const int f = next(k); f >= 0) IO::prefetch(sys_view(p, f, a.bp.vstride), n0, lane);
         IO::load_half(w, n, half, own);
         hops(kEO ? aside(w) : w, false, o);
         const float M = 4.f * rw + s.mass[k], c = kEO ? 0.5f / M : -0.5f;
@@ -609,6 +631,11 @@ __global__ void __launch_bounds__(MAXT, 1)
         const VI w = sys_view(t, s.sys[k], a.bp.vstride);
         const VecP32q<12> rs = sys_view(r, s.sys[k], a.bp.sstride);
         float o[12], own[12], rv[12];
+        if constexpr (kFetch)
+          if (const int f = next(k); f >= 0) {
+            IO::prefetch(sys_view(t, f, a.bp.vstride), n0, lane);
+            RO::prefetch(sys_view(r, f, a.bp.sstride), n0, lane);
+          }
         RO::load_half(rs, n, half, rv);
         IO::load_half(w, n, half, own);
         hops(kEO ? aside(w) : w, true, o);
@@ -632,6 +659,12 @@ __global__ void __launch_bounds__(MAXT, 1)
       const VI w = sys_view(p, s.sys[k], a.bp.vstride);
       const VecP32q<12> xs = sys_view(x, s.sys[k], a.bp.sstride);
       float pv[12], xv[12], rv[12];
+      if constexpr (kFetch)
+        if (const int f = next(k); f >= 0) {
+          IO::prefetch(sys_view(p, f, a.bp.vstride), n0, lane);
+          RO::prefetch(sys_view(x, f, a.bp.sstride), n0, lane);
+          RO::prefetch(sys_view(r, f, a.bp.sstride), n0, lane);
+        }
       IO::load_half(w, n, half, pv);
       RO::load_half(xs, n, half, xv);
       RO::load_half(sys_view(r, s.sys[k], a.bp.sstride), n, half, rv);
