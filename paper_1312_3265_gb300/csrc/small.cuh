@@ -197,15 +197,19 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, nt = gridDim.x;
   const unsigned long long tag = (unsigned long long)epoch << 32;
   unsigned long long* slots = a.slots + (size_t)(PHASE - 1) * a.boxes * nt * nt * 2;
-  // The block's stores, before any of its words: by every warp that may post
-  // one, whichever of its systems still run.
-  if ((int)(threadIdx.x >> 5) < share) fence_gpu();
+  // The block's stores, before any of its words: by every warp that posts, before
+  // its first word, whichever of its systems that is of.  (After the sum: the
+  // stores drain meanwhile; a fence before it cost 0.25 us an exchange.)
+  bool fenced = false;
   for (int t = threadIdx.x >> 5; t < share; t += nw) {
     if (!s.on[t]) continue;
     double v = s.wsum[t][0];
     for (int w = 1; w < nw; ++w) v += s.wsum[t][w];
+    if (!fenced) fence_gpu();
+    fenced = true;
     const unsigned long long hi = tag | (unsigned)__double2hiint(v), lo = tag | (unsigned)__double2loint(v);
-    for (int i = lane; i < nt; i += 32) st_relaxed(slots + ((box(a, s, t) * nt + i) * nt + blockIdx.x) * 2, hi, lo);
+    unsigned long long* w = slots + (box(a, s, t) * nt * nt + blockIdx.x) * 2;
+    for (int i = lane; i < nt; i += 32) st_relaxed(w + (size_t)i * nt * 2, hi, lo);
   }
   int n = 0;
   for (int t = threadIdx.x >> 5; t < share; t += nw) {
@@ -236,10 +240,10 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
   }
   fence_gpu();
   __syncthreads();
-  if (!s.ok) return false;  // (the sums are incomplete)
-  // one thread a system: the divisions of all systems at once
+  // one thread a system: the divisions of all systems at once (after a wait that
+  // gave up, of incomplete sums: not recorded, and the states stay in the block)
   RedBuf rb = a.rb;
-  if (blockIdx.x) rb.hist = nullptr;
+  if (blockIdx.x || !s.ok) rb.hist = nullptr;
   for (int t = threadIdx.x; t < share; t += blockDim.x) {
     if (!s.on[t]) continue;
     SysState& st = s.st[t];
@@ -253,7 +257,7 @@ __device__ __forceinline__ bool exchange(const SmallArgs& a, SmallShared& s, int
     if (st.status != ST_RUNNING) s.on[t] = 0;
   }
   __syncthreads();
-  return true;
+  return s.ok != 0;
 }
 
 // The group's part of the list -> shared memory; returns its size (systems).
@@ -573,8 +577,8 @@ __global__ void __launch_bounds__(MAXT, 1)
   // 46.1 / 43.7, 12^3x16 56.7 / 53.3; below, 8^4 13.2 / 13.5, 12^3x16 with 12
   // systems 15.75 / 15.79.  FP16 storage (half the bytes) and the even-odd
   // operator (its scratch is read, too) gain less than they lose: 36.2 / 37.8 and
-  // 61.6 / 62.5.
-  constexpr bool kFetch = !kEO && std::is_same<VI, VecP32q<12>>::value;
+  // 61.6 / 62.5.  (The wide form holds a system a block: it has no next one.)
+  constexpr bool kFetch = MAXT > kSmallWide && !kEO && std::is_same<VI, VecP32q<12>>::value;
   const int n0 = nn - (lane & 15);
   auto next = [&](int k) {
     return kFetch && a.fetch && k + 1 < share && n0 < V && s.on[k + 1] ? s.sys[k + 1] : -1;
