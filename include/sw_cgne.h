@@ -213,7 +213,10 @@ int cgne_solve_noalloc(const sw_lattice* lat, int op, const void* U, const void*
  *   Mixed-precision solves on lattices that a few hundred warps hold (at 152
  *   SMs: Wilson up to 29184 sites, even-odd twice that, staggered Wilson
  *   14592) run up to 512 iterations in one launch instead (a server's engine 32
- *   or more, by how many systems share the blocks).
+ *   or more, by how many systems share the blocks).  There the launch-per-kernel
+ *   settings -- SW_PARAM_CHUNK, _NS_SW, _NS_WILSON, _GRAPHS, _GROUP_FAST,
+ *   _PERSISTENT and _WILSON_LEAN -- have no effect on a solve, unless the device
+ *   refuses the cooperative launch and the solve goes on with those kernels.
  * SW_PARAM_RELIABLE_DELTA: mixed precision only; the FP32 correction is
  *   folded into the FP64 solution and r = b - A x recomputed in FP64 when the
  *   iterated |r| falls below delta times its maximum since the last such
@@ -322,8 +325,11 @@ int sw_autotune_layout(const sw_lattice* lat, int op, const void* U, const void*
  * systems the launch computed -- and bytes 0.  The stencil classes carry the
  * same flop count besides their bytes.  Every launch of a class while
  * profiling is enabled -- timed or not, graph replays included -- is counted
- * as "issued" (sw_profile_issued), so the time a class takes in a solve is
- * its mean time per timed launch times its issued launches.
+ * as "issued" (sw_profile_issued), so the mean time per timed launch times
+ * the issued launches is the time a class takes by itself.  The solve may take
+ * less: of larger batches the chunks that are not timed run as two halves side
+ * by side (a launch of each half counts as one), and reliable updates run beside
+ * iterations.
  * The one-launch iterations of small lattices (SW_PARAM_CHUNK above) have no
  * k1, k2 and k3 launches to time; their FP64 classes are recorded as always.
  * Process-wide and thread-safe; disabled by default. */
@@ -338,7 +344,7 @@ int sw_measure_fp64_peak(double* tflops, void* stream);
 long long sw_kernel_launches(void);
 
 /* Device workspace cache (no counterpart in the paper).  The solves, the
- * server and the autotuners take their device workspace from one
+ * transport build, the server and the autotuners take their device workspace from one
  * stream-ordered memory pool per device, which keeps freed blocks for the
  * next call (so a solve does not map its workspace anew).
  * sw_workspace_reserved: device bytes the pool of the current device holds,
