@@ -33,9 +33,10 @@
 //
 // An iteration of one system takes 12-14 us, of which the hops are 4, the FP64
 // sums and divisions 3-4 and the fences and inboxes 5.  Measured against the
-// kernels of larger lattices (a solve to 1e-10, same updates): one system, 8^4
-// staggered Wilson 2.87 -> 1.04 ms, 6x10x12x14 Wilson 5.40 -> 2.30; 48 Wilson
-// systems on 8^4 15.0 -> 14.5, on 6x10x12x14 30.7 -> 29.5.
+// kernels of larger lattices on whole chunks: one system to 1e-10, 8^4 staggered
+// Wilson 2.87 -> 1.0 ms, 6x10x12x14 Wilson 5.40 -> 2.2; 12 systems gain 1.04-2.2;
+// 48 are near parity (their FP64 updates run alone here), Wilson to 1e-8: 8^4 13.4
+// / 13.2 ms, 6x10x12x14 26.5 / 26.5, 12^4 41.9 / 43.5, 12^3x16 54.3 / 53.2.
 //
 // The tiles of the reductions depend on the volume only, so a system's
 // results are the same alone and in any batch.
